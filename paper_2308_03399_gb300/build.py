@@ -1,6 +1,6 @@
 """Build libsv.so (CUDA kernels + C++ runtime) in-tree for sm_103a with nvcc.
 
-The two translation units compile in parallel; the result lands in
+The translation units compile in parallel; the result lands in
 paper_2308_03399_gb300/_build/libsv.so.  Nothing is installed elsewhere.
 """
 from __future__ import annotations
@@ -14,8 +14,10 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libsv.so")
 SOURCES = ["sv_kernels.cu", "sv_reg_c64.cu", "sv_reg_c64x.cu", "sv_reg_c128.cu", "sv_runtime.cu", "sv_noalloc.cu",
+           "sv_resident.cu", "sv_resident_c128.cu",
            "sv_mlp.cu", "sv_dm.cu"]
-HEADERS = ["sv_internal.h", "sv_sample.cuh", os.path.join("..", "..", "include", "sv.h"), "sv_common.cuh", "sv_pass_reg.cuh", "sv_pass_whole.cuh"]
+HEADERS = ["sv_internal.h", "sv_sample.cuh", os.path.join("..", "..", "include", "sv.h"), "sv_common.cuh", "sv_pass_reg.cuh", "sv_pass_whole.cuh",
+           "sv_resident.cuh", "sv_resident.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

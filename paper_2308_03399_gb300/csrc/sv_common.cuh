@@ -126,7 +126,7 @@ template <int K> __device__ __forceinline__ void sorted_pos(const int32_t* pos, 
 // the monomial structure of a 4x4 matrix m (row-major), or 0 when it is not
 // monomial; phases go to ph[0..3]
 template <class T>
-__device__ __forceinline__ int mono_info(const T* m, T* ph) {
+__host__ __device__ __forceinline__ int mono_info(const T* m, T* ph) {
     int pi[4];
     for (int q = 0; q < 4; ++q) {
         pi[q] = -1;

@@ -1,0 +1,763 @@
+// Resident runs: a whole circuit for one state per CTA, the state in shared
+// memory from |0...0> to the final sample (k_resident).
+//
+// What bounds the pass-by-pass form for small registers is not bandwidth but
+// the chain of launches: a state of 8 KB to 128 KB gives a pass one group of
+// 16 amplitudes per lane or less, and every pass then costs one branch setup
+// and one L2 round trip for all of the chip.  Here the same passes run back
+// to back inside one kernel.  A CTA owns one state (one shot) at a time and
+// takes the next when it is done, so CTAs on an SM sit in different passes
+// and hide each other's latency chains and barriers.
+//
+// The pass sequence is the one the scheduler recorded, encoded as a program
+// of blocks in the integer pool (sv_resident.h).  Every amplitude goes
+// through the arithmetic of the register pass kernel in the same order
+// (stage by stage, or the folded matrix where the pass was folded), so
+// complex64 states are the same to the last bit.
+//
+// The stage code is kept small on purpose: CTAs sit in different stages, so
+// the instruction cache sees all of it at once.  (A first version that held
+// the twelve register layouts of a two-qubit gate, as the pass kernel does,
+// took 25k to 75k clocks a pass, most of it instruction fetch.)  A stage
+// block therefore has its dense stages on group bits 0 and 1 only, the
+// shared-memory addressing bringing any pair of qubits there, and a folded
+// pass is composed by dynamic indexing.
+//
+// Blocks come in batches of up to `mb` (only the last of a batch may end in a
+// reduction, so the choices of all of them are known): warp w turns block w
+// of the batch into a list of active stages, or its folded matrix, all warps
+// then apply the blocks one after another, and warp 0 decides the reduction.
+// The next batch's blocks are on their way to shared memory (cp.async)
+// meanwhile.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "sv_common.cuh"
+#include "sv_pass_reg.cuh"
+#include "sv_resident.h"
+
+namespace sv {
+
+namespace {
+
+// CTA shapes: registers for 20 complex64 or 12 complex128 warps per SM
+template <class R, int NT> struct ResCta;
+template <> struct ResCta<float, 128> { static constexpr int min_blocks = 5; };
+template <> struct ResCta<float, 512> { static constexpr int min_blocks = 1; };
+template <> struct ResCta<double, 128> { static constexpr int min_blocks = 3; };
+template <> struct ResCta<double, 256> { static constexpr int min_blocks = 1; };
+
+// Shared-memory index of amplitude a: the high bits are folded into the low
+// four, so that 16 lanes whose group indices differ in four address bits of
+// different residues mod 4 touch 16 different 8-byte banks.  Linear over
+// GF(2): swz(a ^ b) = swz(a) ^ swz(b).
+__device__ __forceinline__ int swz(int a) { return a ^ ((a >> 4) & 15) ^ ((a >> 8) & 15) ^ ((a >> 12) & 15); }
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// float-float sum of two pairs (TwoSum of the high words, renormalised)
+__device__ __forceinline__ float2 ff_add(float2 a, float2 b) {
+    const float s = __fadd_rn(a.x, b.x);
+    const float bp = __fsub_rn(s, a.x);
+    float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bp)), __fsub_rn(b.x, bp));
+    e = __fadd_rn(e, __fadd_rn(a.y, b.y));
+    const float hi = __fadd_rn(s, e);
+    return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, s)));
+}
+__device__ __forceinline__ double ff_add(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 shfl_xor2(float2 a, int o) {
+    return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+}
+__device__ __forceinline__ double shfl_xor2(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+template <class A> __device__ __forceinline__ A warp_total(A a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a = ff_add(a, shfl_xor2(a, o));
+    return a;
+}
+__device__ __forceinline__ float2 acc_pair(const Acc<float>& a) { return make_float2(a.hi, a.lo); }
+__device__ __forceinline__ double acc_pair(const Acc<double>& a) { return a.s; }
+__device__ __forceinline__ float2 sum_pair(const svs::Sum<float>& a) { return make_float2(a.hi, a.lo); }
+__device__ __forceinline__ double sum_pair(const svs::Sum<double>& a) { return a.s; }
+
+// Diagonal forms: |v|^2 of a group's amplitudes into the bins of the reduced
+// qubits (group bit 0, or bits 0 and 1).  A register pass over w qubits adds
+// the 2^(w - k) amplitudes of one of its groups that share a bin in R and
+// then once to the compensated accumulator; `run` = 2^(w - k) keeps those
+// sums (the pass's other qubits are the next group bits, in order).
+template <class R, int K>
+__device__ __forceinline__ void res_diag(const typename Cplx<R>::T* v, int run, Acc<R>* acc) {
+#pragma unroll
+    for (int idx = 0; idx < (1 << K); ++idx) {
+        R q = 0;
+#pragma unroll
+        for (int m = 0; m < (16 >> K); ++m) {
+            const int e = idx | (m << K);
+            q += v[e].x * v[e].x + v[e].y * v[e].y;
+            if (((m + 1) & (run - 1)) == 0) {
+                acc[idx].add(q);
+                q = 0;
+            }
+        }
+    }
+}
+
+// one selection by a whole warp: lane r < R holds the probability of outcome
+// r; the running sums, the integer thresholds and the fallback are those of
+// select_k
+__device__ __forceinline__ int warp_select(double p, int R, uint64_t k53) {
+    const int lane = threadIdx.x & 31;
+    double c = lane < R ? p : 0.0;
+    for (int o = 1; o < R; o <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, c, o);
+        if (lane >= o) c += y;
+    }
+    const double prev = __shfl_up_sync(0xffffffffu, c, 1);
+    unsigned m = __ballot_sync(0xffffffffu, lane < R && k53 < cum_threshold(c));
+    if (m) return __ffs(m) - 1;
+    m = __ballot_sync(0xffffffffu, lane < R && c > (lane ? prev : 0.0));
+    return m ? 31 - __clz(m) : R - 1;
+}
+
+// 1 / sqrt(p) of a chosen outcome.  complex64 rounds it to float32 before
+// use, so the float64 reciprocal square root (within an ulp) gives the same
+// factor in a fraction of the float64-pipe time of a root and a division.
+template <class R> __device__ __forceinline__ double res_scale(double p) {
+    return sizeof(R) == 4 ? rsqrt(p) : 1.0 / sqrt(p);
+}
+
+// history of a shot: a sum of one mixed word per (op, outcome), so that two
+// shots with equal words took the same outcomes
+__device__ __forceinline__ unsigned long long hist_word(uint32_t op, int sel) {
+    unsigned long long x = ((unsigned long long)op << 32 | (uint32_t)sel) + 0x9E3779B97F4A7C15ull;
+    x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
+    x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
+    return x ^ (x >> 31);
+}
+
+}  // namespace
+
+// Folded pass (complex64): the active stages composed on the 16 unit vectors,
+// one warp.  Column c of the matrix belongs to lanes c and c + 16, which
+// take half of the row pairs (or quads) of a stage each; the arithmetic is
+// that of the register stages on one group.
+// Work matrix: rows r and r + 1 of column c side by side, so that the dense
+// product reads two entries with one 128-bit load.
+constexpr int FOLD_LD = 17;  // columns of a row pair, padded (bank spread)
+__device__ __forceinline__ int fold_at(int r) { return ((r >> 1) * FOLD_LD << 1) | (r & 1); }
+
+// m0 u + m1 w with every rounding spelled out (the contraction that
+// reg_apply1 compiles to: left to itself, the compiler picks another one here)
+__device__ __forceinline__ float2 row2(float2 m0, float2 m1, float2 u, float2 w) {
+    float2 r;
+    r.x = __fmaf_rn(-m1.y, w.y, __fmaf_rn(m1.x, w.x, __fmaf_rn(m0.x, u.x, -__fmul_rn(m0.y, u.y))));
+    r.y = __fmaf_rn(m1.y, w.x, __fmaf_rn(m1.x, w.y, __fmaf_rn(m0.x, u.y, __fmul_rn(m0.y, u.x))));
+    return r;
+}
+
+// cmul as the register stages round it
+__device__ __forceinline__ float2 cmul_rn(float2 a, float2 b) {
+    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+
+static __device__ __noinline__ void res_compose(const int4* act, int cnt, const unsigned char* smem, float2* M) {
+    const int lane = threadIdx.x & 31, c = lane & 15, h = lane >> 4;
+    float2* const col = M + 2 * c;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) col[fold_at(8 * h + r)] = make_float2(8 * h + r == c ? 1.f : 0.f, 0.f);
+    __syncwarp();
+    for (int s = 0; s < cnt; ++s) {
+        const int4 a = act[s];
+        const int j0 = a.w & 15, j1 = (a.w >> 4) & 15;
+        const float2* m = reinterpret_cast<const float2*>(smem + a.y);
+        if (a.x == RA_ONE || a.x == RA_ONE_SHAPED) {
+            const float2 m0 = m[0], m1 = m[1], m2 = m[2], m3 = m[3];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int g = 4 * h + i, r0 = ((g >> j0) << (j0 + 1)) | (g & ((1 << j0) - 1)), r1 = r0 | (1 << j0);
+                const float2 u = col[fold_at(r0)], w = col[fold_at(r1)];
+                float2 x, y;
+                if (a.x == RA_ONE) {
+                    x = row2(m0, m1, u, w);
+                    y = row2(m2, m3, u, w);
+                } else {
+                    const bool diag = (a.z & 3) == 1;
+                    const float2 p = diag ? m0 : m1, q = diag ? m3 : m2, pu = diag ? u : w, qu = diag ? w : u;
+                    if (a.z & 4) {
+                        x = make_float2(p.x * pu.x, p.x * pu.y);
+                        y = make_float2(q.x * qu.x, q.x * qu.y);
+                    } else {
+                        x = cmul_rn(p, pu);
+                        y = cmul_rn(q, qu);
+                    }
+                }
+                col[fold_at(r0)] = x;
+                col[fold_at(r1)] = y;
+            }
+        } else if (a.x == RA_TWO || a.x == RA_MONO) {
+            const int lo = j0 < j1 ? j0 : j1, hi = j0 < j1 ? j1 : j0;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                int g = 2 * h + i;
+                g = ((g >> lo) << (lo + 1)) | (g & ((1 << lo) - 1));
+                g = ((g >> hi) << (hi + 1)) | (g & ((1 << hi) - 1));
+                const int r[4] = {g, g | (1 << j0), g | (1 << j1), g | (1 << j0) | (1 << j1)};
+                float2 o[4];
+                if (a.x == RA_MONO) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int pq = (a.z >> (8 + 2 * q)) & 3;
+                        const float2 u = col[fold_at(g | ((pq & 1) << j0) | ((pq >> 1) << j1))];
+                        o[q] = a.z & 2 ? u : cmul_rn(m[q], u);
+                    }
+                } else {
+                    unsigned long long ap[4], as[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 u = col[fold_at(r[q])];
+                        ap[q] = pk2(u.x, u.y);
+                        as[q] = pk2(u.y, u.x);
+                    }
+                    const ulonglong2* mx = reinterpret_cast<const ulonglong2*>(m);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        unsigned long long acc = 0ull;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const ulonglong2 mm = mx[q * 4 + e];
+                            acc = fma2(mm.x, ap[e], acc);
+                            acc = fma2(mm.y, as[e], acc);
+                        }
+                        o[q] = upk2(acc);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) col[fold_at(r[q])] = o[q];
+            }
+        } else {  // Pauli string or projection: elementwise on rows, moved by a flip mask
+            float2 o[8];
+            const int x = a.x == RA_PAULI ? a.z & 15 : (a.z >> 16) & 15;
+            const float sc = a.x == RA_PAULI ? 0.f : *reinterpret_cast<const float*>(smem + a.y);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int e = 8 * h + i;
+                float2 t = col[fold_at(e ^ x)];
+                if (a.x == RA_PAULI) {
+                    if ((a.z >> 4) & 1) t = make_float2(t.y, -t.x);
+                    if ((a.z >> (8 + e)) & 1) t = make_float2(-t.x, -t.y);
+                } else if ((a.z >> (e ^ x)) & 1) {
+                    t = make_float2(t.x * sc, t.y * sc);
+                } else {
+                    t = make_float2(0.f, 0.f);
+                }
+                o[i] = t;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) col[fold_at(8 * h + i)] = o[i];
+        }
+        __syncwarp();
+    }
+}
+
+// With at most FOLD_SPARSE nonzero entries in every row, the composed matrix
+// becomes a table: entry k of row r (ascending columns, the order of the
+// dense product's sums; skipped terms are exact zeros) at tab[16 k + r] as
+// (swizzled offset of its amplitude, re, im).  Returns the entries per row;
+// 16: dense, read from the work matrix.
+constexpr int FOLD_SPARSE = 4;
+
+static __device__ __noinline__ int res_table(const float2* M, const int32_t* so, float4* tab) {
+    const int lane = threadIdx.x & 31, r = lane & 15;
+    const float2* row = M + fold_at(r);
+    unsigned nz = 0;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        const float2 m = row[2 * c];
+        nz |= (m.x != 0.f || m.y != 0.f ? 1u : 0u) << c;
+    }
+    int K = __popc(nz);
+    for (int o = 8; o > 0; o >>= 1) K = max(K, __shfl_xor_sync(0xffffffffu, K, o));
+    if (K > FOLD_SPARSE) return 16;
+    for (int k = 0; k < K; ++k) {
+        const int c = nz ? __ffs(nz) - 1 : 0;
+        const float2 m = nz ? row[2 * c] : make_float2(0.f, 0.f);
+        nz &= nz - 1;
+        const int off = (c & 1 ? so[0] : 0) ^ (c & 2 ? so[1] : 0) ^ (c & 4 ? so[2] : 0) ^ (c & 8 ? so[3] : 0);
+        if (lane < 16) tab[16 * k + r] = make_float4(__int_as_float(off), m.x, m.y, 0.f);
+    }
+    return K;
+}
+
+template <class R, int NT>
+__global__ void __launch_bounds__(NT, (ResCta<R, NT>::min_blocks)) k_resident(DevBatch d, const __grid_constant__ ResDesc p) {
+    using T = typename Cplx<R>::T;
+    using A = typename AccSlot<R>::T;
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ int n_act[RES_MAX_BATCH];  // active stages of a block; for a folded one, entries per row
+    __shared__ unsigned long long clb_sh, hist_sh;
+    __shared__ int pset_sh;
+    const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nth >> 5;
+    const int dimp = 1 << p.np, free_bits = p.np - 4, groups = 1 << free_bits;
+    const int mb = p.mb, slots = 2 * mb;
+    T* const st = reinterpret_cast<T*>(smem);
+    int32_t* const blks = reinterpret_cast<int32_t*>(st + dimp);
+    int4* const acts = reinterpret_cast<int4*>(blks + slots * p.block_words);
+    float4* const tabs = reinterpret_cast<float4*>(acts + mb * p.max_stages);
+    float4* const works = tabs + (p.folds ? mb * 16 * FOLD_SPARSE : 0);
+    unsigned char* const brm = reinterpret_cast<unsigned char*>(works + (p.folds ? mb * 8 * FOLD_LD : 0));
+    double* const scale_col = reinterpret_cast<double*>(brm + mb * p.br_bytes);
+    A* const redw = reinterpret_cast<A*>(scale_col + MAX_PEND);
+    double* const fin = reinterpret_cast<double*>(redw + nw * MAX_RED);
+    int32_t* const sel_col = reinterpret_cast<int32_t*>(fin + RES_MAX_FINAL_CHUNKS);
+    uint8_t* const rows = reinterpret_cast<uint8_t*>(sel_col + MAX_PEND);
+    const int2* const index = reinterpret_cast<const int2*>(d.ipool + p.index_off);
+    const int2* const batches = reinterpret_cast<const int2*>(d.ipool + p.batch_off);  // first block, blocks
+    const int n_states = d.ctl[CTL_NBR];
+
+    // warp w: start the copy of block bt.x + w of a batch
+    auto copy_blocks = [&](int2 bt) {
+        if (warp < bt.y) {
+            const int i = bt.x + warp;
+            const int2 ent = index[i];
+            int32_t* dst = blks + (i % slots) * p.block_words;
+            const int32_t* src = d.ipool + ent.x;
+            for (int w = 4 * lane; w < ent.y; w += 128) cp_async16(dst + w, src + w);
+        }
+        cp_commit();
+    };
+
+    // one warp: the active stages of block i (number q of its batch), in op
+    // order, for this state
+    auto prepare = [&](int i, int q) {
+        const int32_t* B = blks + (i % slots) * p.block_words;
+        int4* act = acts + q * p.max_stages;
+        unsigned char* br = brm + q * p.br_bytes;
+        const int n = B[RB_NSTAGES];
+        const uint64_t clb = clb_sh;
+        int count = 0;
+        for (int s0 = 0; s0 < n; s0 += 32) {
+            const int s = s0 + lane;
+            bool on = false;
+            int4 r = make_int4(0, 0, 0, 0);
+            // per-branch matrix: source entries, qubits, scale
+            const T* src = nullptr;
+            double scale = 1.0;
+            int br_k = 0;
+            if (s < n) {
+                const int32_t* S = B + RB_STAGES + RS_WORDS * s;
+                const int w0 = S[0], kind = w0 & 15, k = (w0 >> 4) & 15, pos = S[1];
+                on = true;
+                if ((w0 >> 10) & 1) on = (int)((clb >> ((w0 >> 12) & 63)) & 1) == ((w0 >> 11) & 1);
+                r.w = pos;
+                if (kind == ST_DENSE) {
+                    r.z = B[S[5]];
+                    r.x = k == 1 ? (r.z ? RA_ONE_SHAPED : RA_ONE) : (r.z ? RA_MONO : RA_TWO);
+                    r.y = (int)(reinterpret_cast<const unsigned char*>(B + S[3]) - smem);
+                } else if (kind == ST_DENSE_BR) {
+                    r.y = (int)(br + S[6] - smem);
+                    br_k = k;
+                    if ((w0 >> 20) & 1) {  // the shot's parameter set, from the constant pool
+                        src = reinterpret_cast<const T*>(reinterpret_cast<const R*>(d.pool) + S[3] +
+                                                         (int64_t)pset_sh * S[4]);
+                        r.z = d.ipool[S[5] + pset_sh];
+                    } else {
+                        const int sel = sel_col[S[2]];
+                        scale = scale_col[S[2]];
+                        src = reinterpret_cast<const T*>(B + S[3] + sel * S[4]);
+                        r.z = B[S[5] + sel];
+                    }
+                    r.x = k == 1 ? (r.z ? RA_ONE_SHAPED : RA_ONE) : (r.z ? RA_MONO : RA_TWO);
+                } else if (kind == ST_PAULI_BR) {
+                    const int sel = (w0 >> 9) & 1 ? rows[S[2]] : sel_col[S[2]];
+                    const int packed = B[S[3] + sel];
+                    if ((packed & 0xff) == 0) {
+                        on = false;
+                    } else {
+                        const int xm = packed & 15, zm = (packed >> 4) & 15, ny = (packed >> 8) & 3;
+                        int xg = 0, zg = 0;
+                        for (int j = 0; j < k; ++j) {
+                            const int b = 1 << ((pos >> (4 * j)) & 15);
+                            if ((xm >> j) & 1) xg |= b;
+                            if ((zm >> j) & 1) zg |= b;
+                        }
+                        int sign = 0;
+                        for (int e = 0; e < 16; ++e)
+                            if ((((ny >> 1) & 1) ^ (__popc(zg & e) & 1)) != 0) sign |= 1 << e;
+                        r.x = RA_PAULI;
+                        r.z = xg | ((ny & 1) << 4) | (sign << 8);
+                    }
+                } else {  // ST_PROJ_BR
+                    const int sel = sel_col[S[2]];
+                    int keep = 0, xr = 0;
+                    for (int e = 0; e < 16; ++e) {
+                        int o = 0;
+                        for (int j = 0; j < k; ++j) o |= ((e >> ((pos >> (4 * j)) & 15)) & 1) << j;
+                        if (o == sel) keep |= 1 << e;
+                    }
+                    if ((w0 >> 8) & 1)
+                        for (int j = 0; j < k; ++j)
+                            if ((sel >> j) & 1) xr |= 1 << ((pos >> (4 * j)) & 15);
+                    *reinterpret_cast<R*>(br + S[6]) = (R)scale_col[S[2]];
+                    r.x = RA_PROJ;
+                    r.y = (int)(br + S[6] - smem);
+                    r.z = keep | (xr << 16);
+                }
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, on);
+            if (on) act[count + __popc(m & ((1u << lane) - 1u))] = r;
+            count += __popc(m);
+            // a branch's own matrices: entries over the lanes, times the scale
+            unsigned mb = __ballot_sync(0xffffffffu, on && src != nullptr);
+            while (mb) {
+                const int l = __ffs(mb) - 1;
+                mb &= mb - 1;
+                const T* ls = reinterpret_cast<const T*>(__shfl_sync(0xffffffffu, (unsigned long long)src, l));
+                const R sc = (R)__shfl_sync(0xffffffffu, scale, l);
+                const int off = __shfl_sync(0xffffffffu, r.y, l), code = __shfl_sync(0xffffffffu, r.x, l);
+                const int lk = __shfl_sync(0xffffffffu, br_k, l);
+                const int ne = code == RA_MONO ? 4 : 1 << (2 * lk);
+                if (lane < ne) {
+                    T mm = ls[lane];
+                    mm.x *= sc;
+                    mm.y *= sc;
+                    if (sizeof(T) == 8 && code == RA_TWO)
+                        reinterpret_cast<ulonglong2*>(smem + off)[lane] =
+                            make_ulonglong2(pk2((float)mm.x, (float)mm.x), pk2(-(float)mm.y, (float)mm.y));
+                    else
+                        reinterpret_cast<T*>(smem + off)[lane] = mm;
+                }
+            }
+        }
+        __syncwarp();
+        if constexpr (sizeof(T) == 8) {
+            if (B[RB_FOLD]) {
+                if (count > 0) {
+                    float2* M = reinterpret_cast<float2*>(works + q * 8 * FOLD_LD);
+                    res_compose(act, count, smem, M);
+                    count = res_table(M, B + RB_SO, tabs + q * 16 * FOLD_SPARSE);
+                }
+            }
+        }
+        if (lane == 0) n_act[q] = count;
+        __syncwarp();
+    };
+
+    const int2 none = make_int2(0, 0), first = p.n_batches > 0 ? batches[0] : none;
+
+    for (int state = blockIdx.x; state < n_states; state += gridDim.x) {
+        const uint32_t shot = (uint32_t)state;  // batch mode: shot s is branch s in slot s
+        const uint64_t gs = d.shot_base + shot;
+        copy_blocks(first);
+        if (tid == 0) {
+            clb_sh = 0;
+            pset_sh = d.br_pset[state];
+            hist_sh = p.hist ? hist_word(0xffffffffu, d.br_pset[state]) : 0ull;
+        }
+        for (int j = tid; j < dimp; j += nth) {
+            T z;
+            z.x = j == 0 ? (R)1 : (R)0;
+            z.y = 0;
+            st[j] = z;
+        }
+        // the shot's choice of every Pauli op: state-independent, drawn first
+        unsigned long long hsum = 0;
+        for (int q = tid; q < p.n_rows; q += nth) {
+            const int32_t* e = d.ipool + p.row_table + (int64_t)PRE_WORDS * q;
+            const uint32_t op = (uint32_t)e[0];
+            const int sel = select_k(philox_k53(d.seed, gs, op), reinterpret_cast<const uint64_t*>(d.ipool + e[2]),
+                                     reinterpret_cast<const double*>(d.ipool + e[3]), e[1]);
+            rows[q] = (uint8_t)sel;
+            hsum += hist_word(op, sel);
+        }
+        __syncthreads();
+        if (p.hist && hsum) atomicAdd(&hist_sh, hsum);
+        int2 bt = first, nxt = p.n_batches > 1 ? batches[1] : none;
+        for (int t = 0, q = 0; t < p.n_batches;) {
+            if (q == 0) {
+                if (warp < bt.y) {
+                    cp_wait0();
+                    __syncwarp();
+                    prepare(bt.x + warp, warp);
+                }
+                __syncthreads();
+                copy_blocks(nxt);
+            }
+            const int i = bt.x + q;
+            const int32_t* B = blks + (i % slots) * p.block_words;
+            const int rw = B[RB_RED], red_kind = rw & 15, red_k = (rw >> 4) & 15, red_R = (rw >> 8) & 31;
+            const bool red = red_kind != RED_NONE;
+            Acc<R> acc[REG_MAX_RED];
+#pragma unroll
+            for (int r = 0; r < REG_MAX_RED; ++r) acc[r].zero();
+            // swizzled offsets of the group-number bits, two to a word
+            int sfw[5];
+#pragma unroll
+            for (int j = 0; j < 5; ++j) sfw[j] = B[RB_SF + j];
+            auto group_base = [&](int g) {
+                int b = 0;
+#pragma unroll
+                for (int j = 0; j < 5; ++j) {
+                    b ^= g & (1 << (2 * j)) ? sfw[j] & 0xffff : 0;
+                    b ^= g & (2 << (2 * j)) ? (int)((unsigned)sfw[j] >> 16) : 0;
+                }
+                return b;
+            };
+            const int so0 = B[RB_SO], so1 = B[RB_SO + 1], so2 = B[RB_SO + 2], so3 = B[RB_SO + 3];
+            auto off = [&](int e) {
+                return ((e & 1) ? so0 : 0) ^ ((e & 2) ? so1 : 0) ^ ((e & 4) ? so2 : 0) ^ ((e & 8) ? so3 : 0);
+            };
+            if (sizeof(T) == 8 && B[RB_FOLD]) {
+                if constexpr (sizeof(T) == 8) {
+                    const int K = n_act[q];
+                    const float4* tab = tabs + q * 16 * FOLD_SPARSE;
+                    const float4* M = works + q * 8 * FOLD_LD;
+                    for (int g = tid; K > 0 && g < groups; g += nth) {
+                        const int base = group_base(g);
+                        float2 o[16];
+                        if (K <= FOLD_SPARSE) {
+#pragma unroll
+                            for (int r = 0; r < 16; ++r) o[r] = make_float2(0.f, 0.f);
+                            for (int k = 0; k < K; ++k) {
+#pragma unroll
+                                for (int r = 0; r < 16; ++r) {
+                                    const float4 m = tab[16 * k + r];
+                                    const float2 a = st[base ^ __float_as_int(m.x)];
+                                    o[r].x = fmaf(m.y, a.x, fmaf(-m.z, a.y, o[r].x));
+                                    o[r].y = fmaf(m.y, a.y, fmaf(m.z, a.x, o[r].y));
+                                }
+                            }
+#pragma unroll
+                            for (int r = 0; r < 16; ++r) st[base ^ off(r)] = o[r];
+                        } else {
+#pragma unroll
+                            for (int r = 0; r < 16; ++r) o[r] = st[base ^ off(r)];
+#pragma unroll 1
+                            for (int r = 0; r < 16; r += 2) {
+                                float2 x = make_float2(0.f, 0.f), y = make_float2(0.f, 0.f);
+#pragma unroll
+                                for (int c = 0; c < 16; ++c) {
+                                    const float4 m = M[(r >> 1) * FOLD_LD + c];
+                                    const float2 a = o[c];
+                                    x.x = fmaf(m.x, a.x, fmaf(-m.y, a.y, x.x));
+                                    x.y = fmaf(m.x, a.y, fmaf(m.y, a.x, x.y));
+                                    y.x = fmaf(m.z, a.x, fmaf(-m.w, a.y, y.x));
+                                    y.y = fmaf(m.z, a.y, fmaf(m.w, a.x, y.y));
+                                }
+                                st[base ^ off(r)] = x;
+                                st[base ^ off(r) ^ so0] = y;
+                            }
+                        }
+                    }
+                }
+            } else {
+                const int4* act = acts + q * p.max_stages;
+                const int cnt = n_act[q];
+                const bool touch = cnt > 0 || red_kind == RED_DIAG || red_kind == RED_FORMS;
+                for (int g = tid; touch && g < groups; g += nth) {
+                    const int base = group_base(g);
+                    T v[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) v[e] = st[base ^ off(e)];
+#pragma unroll 1
+                    for (int s = 0; s < cnt; ++s) {
+                        const int4 r = act[s];
+                        const T* m = reinterpret_cast<const T*>(smem + r.y);
+                        if (r.x == RA_ONE_SHAPED) {
+                            if (r.w & 15) reg_apply1_shaped<T, 16, 1>(v, m, r.z);
+                            else reg_apply1_shaped<T, 16, 0>(v, m, r.z);
+                        } else if (r.x == RA_ONE) {
+                            if (r.w & 15) reg_apply1<T, 16, 1>(v, m);
+                            else reg_apply1<T, 16, 0>(v, m);
+                        } else if (r.x == RA_MONO) {
+                            reg_mono<T, 16, 0, 1>(v, r.z, m);
+                        } else if (r.x == RA_TWO) {
+                            if constexpr (sizeof(T) == 8)
+                                reg_apply2_f32x2<16, 0, 1>(reinterpret_cast<float2*>(v),
+                                                           reinterpret_cast<const ulonglong2*>(m));
+                            else
+                                reg_apply2<T, 16, 0, 1>(v, m);
+                        } else if (r.x == RA_PAULI) {
+                            reg_xor_mask<T, 16>(v, r.z & 15);
+                            const bool rot = (r.z >> 4) & 1;
+                            const int sign = r.z >> 8;
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) {
+                                T t = v[e];
+                                if (rot) {
+                                    const R x = t.x;
+                                    t.x = t.y;
+                                    t.y = -x;
+                                }
+                                if ((sign >> e) & 1) {
+                                    t.x = -t.x;
+                                    t.y = -t.y;
+                                }
+                                v[e] = t;
+                            }
+                        } else {
+                            const R sc = m->x;
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) {
+                                if ((r.z >> e) & 1) {
+                                    v[e].x *= sc;
+                                    v[e].y *= sc;
+                                } else {
+                                    v[e].x = 0;
+                                    v[e].y = 0;
+                                }
+                            }
+                            reg_xor_mask<T, 16>(v, (r.z >> 16) & 15);
+                        }
+                    }
+                    if (red_kind == RED_DIAG) {
+                        const int run = B[RB_RUN];
+                        if (red_k == 2) res_diag<R, 2>(v, run, acc);
+                        else res_diag<R, 1>(v, run, acc);
+                    } else if (red_kind == RED_FORMS) {
+                        reg_forms1<R, 16, 0>(v, reinterpret_cast<const T*>(B + B[RB_COEF]), red_R, acc);
+                    }
+                    if (cnt > 0)
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) st[base ^ off(e)] = v[e];
+                }
+            }
+            if (red) {
+                const int nv = red_kind == RED_DIAG ? 1 << red_k : red_R;  // values reduced over the state
+                if (red_kind == RED_BINS) {
+                    // a warp owns an outcome: its amplitudes, one compensated
+                    // addition each, in a fixed order
+                    __syncthreads();
+                    const int rp = B[RB_RPOS];
+                    for (int o = warp; o < red_R; o += nw) {
+                        Acc<R> a;
+                        a.zero();
+                        for (int g = lane; g < groups; g += 32) {
+                            const int base = group_base(g);
+                            for (int e = 0; e < 16; ++e) {
+                                int b = 0;
+                                for (int j = 0; j < red_k; ++j) b |= ((e >> ((rp >> (4 * j)) & 15)) & 1) << j;
+                                if (b != o) continue;
+                                const T x = st[base ^ off(e)];
+                                a.add(x.x * x.x + x.y * x.y);
+                            }
+                        }
+                        const A t = warp_total(acc_pair(a));
+                        if (lane == 0) redw[o] = t;
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < REG_MAX_RED; ++r) {
+                        if (r >= nv) break;
+                        const A t = warp_total(acc_pair(acc[r]));
+                        if (lane == 0) redw[warp * MAX_RED + r] = t;
+                    }
+                }
+                __syncthreads();
+                if (warp == 0) {
+                    // totals (lane r: value r), then the probabilities
+                    double val = 0.0;
+                    if (lane < nv) {
+                        A t = redw[lane];
+                        if (red_kind != RED_BINS)
+                            for (int w = 1; w < nw; ++w) t = ff_add(t, redw[w * MAX_RED + lane]);
+                        val = acc_get(t);
+                    }
+                    double pr = val;
+                    if (red_kind == RED_DIAG) {
+                        const double* W = reinterpret_cast<const double*>(B + B[RB_COEF]) + (lane < red_R ? lane << red_k : 0);
+                        pr = 0.0;
+                        for (int r = 0; r < nv; ++r) pr += W[r] * __shfl_sync(0xffffffffu, val, r);
+                    }
+                    const int32_t* D = B + B[RB_DECIDE];
+                    const int kind = D[RD_KIND], nR = D[RD_R], r2 = D[RD_R2];
+                    double ph = pr;  // the head op's probabilities, lane r: outcome r
+                    if (kind == DEC_KRAUS_J1) {
+                        ph = 0.0;
+                        const int base = lane < nR ? lane * r2 : 0;
+                        for (int j = 0; j < r2; ++j) ph += __shfl_sync(0xffffffffu, pr, base + j);
+                    }
+                    const int o1 = warp_select(ph, nR, philox_k53(d.seed, gs, (uint32_t)D[RD_OP]));
+                    const double p1 = __shfl_sync(0xffffffffu, ph, o1);
+                    if (lane == 0) {
+                        sel_col[D[RD_PEND]] = o1;
+                        scale_col[D[RD_PEND]] = res_scale<R>(p1);
+                        if (p.hist) hist_sh += hist_word((uint32_t)D[RD_OP], o1);
+                        if (kind == DEC_MEASURE) {
+                            unsigned long long cl = clb_sh;
+                            for (int j = 0; j < D[RD_M]; ++j) {
+                                const int b = (D[RD_CLBITS] >> (8 * j)) & 255;
+                                cl = (cl & ~(1ull << b)) | ((unsigned long long)((o1 >> j) & 1) << b);
+                            }
+                            clb_sh = cl;
+                        }
+                    }
+                    if (kind == DEC_KRAUS_J1) {
+                        // op 2 from p(j | o1) = p_ij / p_i
+                        const double pj = __shfl_sync(0xffffffffu, pr, o1 * r2 + (lane < r2 ? lane : 0)) / p1;
+                        const int o2 = warp_select(pj, r2, philox_k53(d.seed, gs, (uint32_t)D[RD_OP2]));
+                        const double p2 = __shfl_sync(0xffffffffu, pj, o2);
+                        if (lane == 0) {
+                            sel_col[D[RD_PEND2]] = o2;
+                            scale_col[D[RD_PEND2]] = res_scale<R>(p2);
+                            if (p.hist) hist_sh += hist_word((uint32_t)D[RD_OP2], o2);
+                        }
+                    }
+                    __syncwarp();
+                }
+                // the next batch's lists read the choices: a batch of one
+                // block is prepared by the warp that made them
+                if (nxt.y > 1) __syncthreads();
+            } else {
+                __syncthreads();
+            }
+            if (++q == bt.y) {
+                q = 0;
+                ++t;
+                bt = nxt;
+                nxt = t + 1 < p.n_batches ? batches[t + 1] : none;
+            }
+        }
+        __syncthreads();
+
+        // the final state to its slot, and the final sample
+        T* const out = reinterpret_cast<T*>(d.states) + (int64_t)shot * d.dim;
+        const int dim = (int)d.dim;
+        for (int j = tid; j < dim; j += nth) out[j] = st[swz(j)];
+        if (p.has_final) {
+            const int len = dim < 256 ? dim : 256, chunks = dim / len;
+            for (int c = warp; c < chunks; c += nw) {
+                svs::Sum<R> a;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int j = lane * 8 + e;
+                    if (j < len) {
+                        const T x = st[swz(c * len + j)];
+                        a.add_sq(x.x, x.y);
+                    }
+                }
+                const A t = warp_total(sum_pair(a));
+                if (lane == 0) fin[c] = acc_get(t);
+            }
+            __syncthreads();
+            if (warp == 0) {
+                svs::chunk_cum(fin, fin, chunks, 1);
+                __syncwarp();
+                const double u = philox_uniform(d.seed, gs, p.fin_op);
+                double lo, hi;
+                const int64_t key = svs::sample_warp<R>(out, dim, chunks, fin, 1, u, &lo, &hi);
+                if (lane == 0) d.keys[shot] = (uint64_t)key;
+            }
+        }
+        if (tid == 0 && p.hist) p.hist[shot] = hist_sh;
+        __syncthreads();  // st, rows and the block ring are free again
+    }
+}
+
+}  // namespace sv

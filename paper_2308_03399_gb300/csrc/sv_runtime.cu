@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <cmath>
 #include <complex>
@@ -25,7 +26,9 @@
 #include <vector>
 
 #include "../../include/sv.h"
+#include "sv_common.cuh"
 #include "sv_internal.h"
+#include "sv_resident.h"
 
 using namespace sv;
 
@@ -60,7 +63,7 @@ struct PreRow {
     double* log_thr;
 };
 
-enum LType { L_INIT, L_RESET, L_PASS, L_DECIDE, L_ALLOC, L_COPY, L_FINAL, L_PREDRAW };
+enum LType { L_INIT, L_RESET, L_PASS, L_DECIDE, L_ALLOC, L_COPY, L_FINAL, L_PREDRAW, L_RESIDENT };
 enum PClass { P_PASS = 0, P_DECIDE, P_ALLOC, P_COPY, P_FINAL, P_INIT, P_OTHER, P_N };
 
 struct Launch {
@@ -70,6 +73,7 @@ struct Launch {
     PassDesc pass;
     DecideDesc dec;
     FinalDesc fin;
+    ResDesc res;  // L_RESIDENT; a0: the passes of its circuit, a1: states
 };
 
 // Philox4x32-10 on the host (plain per-shot mode draws on the host, as the
@@ -196,6 +200,14 @@ struct sv_batch_s {
     int pre_cap = 0;               // rows the device table holds
     std::map<int, int> reg_occ;
     int slot_limit = 0;
+    // resident runs (k_resident): options that shape the pass kernels and
+    // differ from their defaults (one bit per option) keep a run on them
+    uint32_t tuned = 0;
+    bool rec_resident = false;  // the circuit being recorded may become a resident run
+    std::vector<Launch> res_list;
+    uint64_t res_hash = 0, res_gen = 0;
+    double res_bytes = 0;  // states written by resident runs since sv_stats
+    std::map<int, int> term_count, term_count_i;  // terms at a pool / integer-pool offset (recording)
     // parameter sweep (sv_set_param_sets): every shot's parameter set
     int n_psets = 0;
     std::vector<uint32_t> h_pset;
@@ -228,6 +240,7 @@ template <class T> sv_status dalloc(sv_batch b, T** p, size_t count) {
 int pclass(LType t) {
     switch (t) {
     case L_PASS: return P_PASS;
+    case L_RESIDENT: return P_PASS;
     case L_DECIDE: return P_DECIDE;
     case L_PREDRAW: return P_DECIDE;
     case L_ALLOC: return P_ALLOC;
@@ -278,7 +291,7 @@ int pass_grid(sv_batch b, const PassDesc& p) {
 cudaError_t exec_one(sv_batch b, const Launch& L) {
     const int prec = b->prec == SV_C128;
     switch (L.type) {
-    case L_INIT: return launch_init(b->dev, prec, L.a0, b->n_sm * 4, b->stream);
+    case L_INIT: return L.a0 == 0 ? cudaSuccess : launch_init(b->dev, prec, L.a0, b->n_sm * 4, b->stream);
     case L_RESET: return launch_reset(b->dev, L.a0, L.a1, L.a2, b->n_sm * 2, b->stream);
     case L_PASS:
         if (L.pass.whole) return launch_pass_whole(b->dev, L.pass, pass_grid(b, L.pass), b->stream);
@@ -288,8 +301,25 @@ cudaError_t exec_one(sv_batch b, const Launch& L) {
     case L_COPY: return launch_copy(b->dev, prec, b->n_sm * 4, b->stream);
     case L_FINAL: return launch_final(b->dev, prec, L.fin, b->grid_small, b->stream);
     case L_PREDRAW: return launch_predraw(b->dev, L.a0, L.a1, L.a2, b->n_sm * 4, b->stream);
+    case L_RESIDENT: return launch_resident(b->dev, prec, L.res, L.a1, b->n_sm, b->stream);
     }
     return cudaErrorInvalidValue;
+}
+
+int launch_kernels(const Launch& L) {
+    if (L.type == L_INIT && L.a0 == 0) return 0;
+    return L.type == L_FINAL ? 3 : (L.type == L_DECIDE ? 2 : 1);
+}
+
+void count_launch(sv_batch b, const Launch& L) {
+    b->n_launch += launch_kernels(L);
+    if (L.type == L_PASS) {
+        b->n_passes += 1;
+        b->pass_store.push_back(L.pass.store ? 1 : 0);
+    } else if (L.type == L_RESIDENT) {
+        b->n_passes += L.a0;
+        b->res_bytes += (double)L.a1 * (double)b->state_bytes;
+    }
 }
 
 sv_status exec(sv_batch b, const Launch& L) {
@@ -305,11 +335,7 @@ sv_status exec(sv_batch b, const Launch& L) {
         cudaEventRecord(e1, b->stream);
         b->prof_ev.push_back({pclass(L.type), {e0, e1}});
     }
-    b->n_launch += L.type == L_FINAL ? 3 : (L.type == L_DECIDE ? 2 : 1);
-    if (L.type == L_PASS) {
-        b->n_passes += 1;
-        b->pass_store.push_back(L.pass.store ? 1 : 0);
-    }
+    count_launch(b, L);
     return SV_OK;
 }
 
@@ -1121,9 +1147,10 @@ sv_status op_pauli(sv_batch b, uint32_t op, int k, const int* q, int n_terms, co
     // batch mode, whole circuits: the choice of every shot is drawn up front
     // (k_predraw), so the op needs no decide and no pending column
     const bool pre = b->rec && !b->branch && b->predraw &&
-                     (uint64_t)(b->pre_rows.size() + 1) * b->n_shots <= PRE_TABLE_BYTES;
+                     (b->rec_resident || (uint64_t)(b->pre_rows.size() + 1) * b->n_shots <= PRE_TABLE_BYTES);
     if ((st = make_room(b, q, k, 0, !pre))) return st;
     const int off = (int)b->ipool.size();
+    b->term_count_i[off] = n_terms;
     for (int t = 0; t < n_terms; ++t) b->ipool.push_back(pauli_packed(paulis + t * k, k));
     int pend;
     if (pre) {
@@ -1252,6 +1279,7 @@ sv_status op_kraus(sv_batch b, uint32_t op, int k, const int* q, int n_terms, co
     for (int j = 0; j < k; ++j) red.q[j] = q[j];
     push_forms(b, F, k, n_terms, red);
     const int mat_off = (int)b->pool.size();
+    b->term_count[mat_off] = n_terms;
     for (int i = 0; i < 2 * E * n_terms; ++i) b->pool.push_back(kraus[i]);
     if ((st = upload_pool(b))) return st;
     if ((st = emit_reduction(b, red, 2 * n_terms * E))) return st;
@@ -1302,8 +1330,10 @@ sv_status op_kraus_pair(sv_batch b, uint32_t op1, int qa, int n1, const double* 
     red.q[1] = qb;
     push_forms(b, F, 2, n1 * n2, red);
     const int m1 = (int)b->pool.size();
+    b->term_count[m1] = n1;
     for (int i = 0; i < 8 * n1; ++i) b->pool.push_back(k1[i]);
     const int m2 = (int)b->pool.size();
+    b->term_count[m2] = n2;
     for (int i = 0; i < 8 * n2; ++i) b->pool.push_back(k2[i]);
     if ((st = upload_pool(b))) return st;
     if ((st = emit_reduction(b, red, 2 * n1 * n2 * 16))) return st;
@@ -1605,8 +1635,7 @@ sv_status run_plain(sv_batch b, const sv_circuit* c) {
 // the pre-drawn rows of a recorded circuit: their descriptors go to the
 // integer pool, the device table grows to hold them, and the draw is the
 // circuit's first launch
-sv_status finish_predraw(sv_batch b, std::vector<Launch>& launches) {
-    const int n = (int)b->pre_rows.size();
+int push_row_table(sv_batch b) {
     const int table = (int)b->ipool.size();
     for (const PreRow& r : b->pre_rows) {
         const uint64_t ls = (uint64_t)(uintptr_t)r.log_sel, lt = (uint64_t)(uintptr_t)r.log_thr;
@@ -1614,6 +1643,12 @@ sv_status finish_predraw(sv_batch b, std::vector<Launch>& launches) {
                                       (int32_t)(uint32_t)(ls >> 32), (int32_t)(uint32_t)lt, (int32_t)(uint32_t)(lt >> 32)};
         b->ipool.insert(b->ipool.end(), w, w + PRE_WORDS);
     }
+    return table;
+}
+
+sv_status finish_predraw(sv_batch b, std::vector<Launch>& launches) {
+    const int n = (int)b->pre_rows.size();
+    const int table = push_row_table(b);
     if (n > b->pre_cap) {
         sv_status st = dalloc(b, &b->dev.pre_sel, (size_t)n * b->n_shots);
         if (st) return st;
@@ -1629,7 +1664,429 @@ sv_status finish_predraw(sv_batch b, std::vector<Launch>& launches) {
     return SV_OK;
 }
 
-sv_status record_circuit(sv_batch b, const sv_circuit* c, std::vector<Launch>& launches) {
+// ---- resident runs (k_resident) ----------------------------------------------
+// A batch-mode circuit whose state fits a CTA's shared memory runs as one
+// launch.  Options that shape the pass kernels (a tile or fusion width, a
+// CTA size, a path, ...) keep the run on those kernels, and so does the log:
+// the logged running sums of batch and shot-branching runs are the same to
+// the last bit, and the resident kernel sums in another order.
+constexpr int RES_MAX_QUBITS_C64 = 14, RES_MAX_QUBITS_C128 = 13;
+
+bool resident_candidate(sv_batch b) {
+    if (b->tuned || b->log || b->branch || b->mode == SV_PLAIN) return false;
+    return b->n <= (b->prec == SV_C128 ? RES_MAX_QUBITS_C128 : RES_MAX_QUBITS_C64);
+}
+
+// one block of a resident program: 32-bit words, matrices in the batch's
+// precision
+struct ResBlock {
+    std::vector<int32_t> w;
+    bool c128;
+    void align(int words) {
+        while (w.size() % words) w.push_back(0);
+    }
+    void f64(double v) {
+        uint64_t u;
+        memcpy(&u, &v, 8);
+        w.push_back((int32_t)(uint32_t)u);
+        w.push_back((int32_t)(uint32_t)(u >> 32));
+    }
+    void real(double v) {
+        if (c128) return f64(v);
+        const float f = (float)v;
+        int32_t u;
+        memcpy(&u, &f, 4);
+        w.push_back(u);
+    }
+};
+
+// entry e of a matrix in the constant pool, as the kernels read it
+double2 pool_entry(sv_batch b, int64_t off, int e) {
+    const double x = b->pool[off + 2 * e], y = b->pool[off + 2 * e + 1];
+    return b->prec == SV_C128 ? make_double2(x, y) : make_double2((double)(float)x, (double)(float)y);
+}
+
+// structure of a one-qubit matrix: 1 diagonal, 2 anti-diagonal, +4 real
+int shape1(const double2* m) {
+    auto z = [](double2 v) { return v.x == 0 && v.y == 0; };
+    int s = z(m[1]) && z(m[2]) ? 1 : (z(m[0]) && z(m[3]) ? 2 : 0);
+    if (s == 1 && m[0].y == 0 && m[3].y == 0) s |= 4;
+    if (s == 2 && m[1].y == 0 && m[2].y == 0) s |= 4;
+    return s;
+}
+
+// The group qubits of a block: `fixed` in this order at group bits 0.., then
+// fillers, chosen so that the other address bits cover every residue mod 4
+// where they can; `order` numbers the groups by those bits, four of different
+// residues first (bank-conflict-free, see res_swz).
+void res_group(const std::vector<int>& fixed, int np, int* gq, std::vector<int>& order) {
+    uint64_t act = 0;
+    for (int q : fixed) act |= 1ull << q;
+    std::vector<int> rest;
+    for (int q = 0; q < np; ++q)
+        if (!((act >> q) & 1)) rest.push_back(q);
+    const int need = 4 - (int)fixed.size(), nr = (int)rest.size();
+    uint64_t best = 0;
+    int best_score = -1;
+    for (uint64_t m = 0; m < (1ull << nr) && best_score < std::min(4, np - 4); ++m) {
+        if (__builtin_popcountll(m) != need) continue;
+        uint64_t fill = 0;
+        int res = 0;
+        for (int j = 0; j < nr; ++j) {
+            if ((m >> j) & 1) fill |= 1ull << rest[j];
+            else res |= 1 << (rest[j] & 3);
+        }
+        if (__builtin_popcount(res) > best_score) {
+            best_score = __builtin_popcount(res);
+            best = fill;
+        }
+    }
+    int n = 0, seen = 0;
+    for (int q : fixed) gq[n++] = q;
+    std::vector<int> later;
+    order.clear();
+    for (int q : rest) {
+        if ((best >> q) & 1) gq[n++] = q;
+        else if (!((seen >> (q & 3)) & 1)) {
+            seen |= 1 << (q & 3);
+            order.push_back(q);
+        } else later.push_back(q);
+    }
+    order.insert(order.end(), later.begin(), later.end());
+}
+
+// one block: stages s0 .. s1 of a recorded pass on group qubits that start
+// with `fixed`, and (dec) the pass's reduction and its decide; false when it
+// holds something k_resident does not run
+bool res_block(sv_batch b, const PassDesc& p, int s0, int s1, const std::vector<int>& fixed, const DecideDesc* dec,
+               int np, ResBlock& B, int* br_bytes) {
+    const bool c128 = b->prec == SV_C128;
+    B.c128 = c128;
+    int gq[4];
+    std::vector<int> order;
+    res_group(fixed, np, gq, order);
+    auto gbit = [&](int pos) {
+        const int q = p.tile_q[pos];
+        for (int j = 0; j < 4; ++j)
+            if (gq[j] == q) return j;
+        return 0;
+    };
+    B.w.assign(RB_STAGES + RS_WORDS * (s1 - s0), 0);
+    B.w[RB_NSTAGES] = s1 - s0;
+    B.w[RB_FOLD] = p.fold;
+    for (int j = 0; j < 4; ++j) B.w[RB_SO + j] = res_swz(1 << gq[j]);
+    for (size_t j = 0; j < order.size(); ++j) B.w[RB_SF + j / 2] |= res_swz(1 << order[j]) << (16 * (j & 1));
+    int br = 0;
+    for (int s = s0; s < s1; ++s) {
+        const Stage& st = p.st[s];
+        int32_t S[RS_WORDS] = {};
+        const bool pset = st.kind == ST_DENSE_BR && st.pend == PEND_PSET;
+        if (st.cond_clbit >= 0 && (st.cond_val < 0 || st.cond_val > 1)) return false;
+        S[0] = st.kind | st.k << 4 | (st.reset ? 1 << 8 : 0) | (st.pre ? 1 << 9 : 0) |
+               (st.cond_clbit >= 0 ? 1 << 10 | st.cond_val << 11 | st.cond_clbit << 12 : 0) | (pset ? 1 << 20 : 0);
+        for (int j = 0; j < st.k; ++j) S[1] |= gbit(st.pos[j]) << (4 * j);
+        S[2] = pset ? 0 : st.pend;
+        if (st.kind == ST_DENSE || st.kind == ST_DENSE_BR) {
+            if (st.k > 2) return false;
+            // a monomial matrix written for bits (1, 0) is rewritten for (0, 1):
+            // bit-swapped row and column indices
+            const bool swap = st.k == 2 && !p.fold && (S[1] & 0xff) == 0x01;
+            const int E = 1 << (2 * st.k);
+            int terms = 1;
+            if (st.kind == ST_DENSE_BR) {
+                auto it = b->term_count.find(st.off);
+                terms = pset ? b->n_psets : (it == b->term_count.end() ? 0 : it->second);
+            }
+            if (terms < 1) return false;
+            // the structure of every term; a per-branch term's phases carry
+            // its scale, so it is never taken as one of unit phases
+            std::vector<int> info(terms);
+            std::vector<std::array<double2, 4>> phs(terms);
+            bool all_mono = st.k == 2;
+            for (int t = 0; t < terms; ++t) {
+                double2 m[16], ph[4] = {};
+                for (int e = 0; e < E; ++e) {
+                    const int r = e >> st.k, c = e & ((1 << st.k) - 1);
+                    auto sw = [&](int i) { return swap ? ((i & 1) << 1) | (i >> 1) : i; };
+                    m[sw(r) << st.k | sw(c)] = pool_entry(b, st.off + (int64_t)t * st.stride, e);
+                }
+                info[t] = st.k == 1 ? shape1(m) : (pset ? 0 : mono_info(m, ph));
+                if (st.k == 2 && st.kind == ST_DENSE_BR) info[t] &= ~2;
+                for (int j = 0; j < 4; ++j) phs[t][j] = ph[j];
+                all_mono = all_mono && info[t];
+            }
+            if (swap && !all_mono) return false;  // the caller keeps dense pairs in order
+            if (swap) S[1] = 0x10;
+            if (pset) {
+                S[3] = st.off;
+                S[4] = st.stride;
+                S[5] = (int)b->ipool.size();
+                b->ipool.insert(b->ipool.end(), info.begin(), info.end());
+            } else {
+                B.align(4);
+                S[3] = (int)B.w.size();
+                const bool expand = st.kind == ST_DENSE && st.k == 2 && !info[0] && !c128;
+                const int entries = all_mono ? 4 : E;
+                S[4] = entries * 2 * (c128 ? 2 : 1);
+                for (int t = 0; t < terms; ++t)
+                    for (int e = 0; e < entries; ++e) {
+                        double2 v = make_double2(0, 0);
+                        if (st.k == 2 && info[t]) {
+                            if (e < 4) v = phs[t][e];
+                        } else {
+                            v = pool_entry(b, st.off + (int64_t)t * st.stride, e);
+                        }
+                        B.real(v.x);
+                        if (expand) {  // (re, re, -im, im) for packed FMAs
+                            B.real(v.x);
+                            B.real(-v.y);
+                        }
+                        B.real(v.y);
+                    }
+                S[5] = (int)B.w.size();
+                B.w.insert(B.w.end(), info.begin(), info.end());
+            }
+            if (st.kind == ST_DENSE_BR) {
+                S[6] = br;
+                br += E * 16;  // complex128 entries, or expanded complex64 ones
+            }
+        } else if (st.kind == ST_PAULI_BR) {
+            auto it = b->term_count_i.find(st.off);
+            if (it == b->term_count_i.end()) return false;
+            S[3] = (int)B.w.size();
+            for (int t = 0; t < it->second; ++t) B.w.push_back(b->ipool[st.off + t]);
+        } else {
+            S[6] = br;
+            br += 16;
+        }
+        memcpy(&B.w[RB_STAGES + RS_WORDS * (s - s0)], S, sizeof(S));
+    }
+    *br_bytes = br;
+    if (!dec) {
+        B.align(4);
+        return true;
+    }
+    B.w[RB_RED] = p.red_kind | p.red_k << 4 | p.red_R << 8;
+    for (int j = 0; j < p.red_k; ++j) B.w[RB_RPOS] |= gbit(p.red_pos[j]) << (4 * j);
+    if (p.red_kind == RED_DIAG) {
+        if (p.red_k > 2 || p.red_R > MAX_RED) return false;
+        B.w[RB_RUN] = p.reg_wp > 0 ? 1 << (p.reg_wp - p.red_k) : 1;
+        B.align(4);
+        B.w[RB_COEF] = (int)B.w.size();
+        const int n = p.red_R << p.red_k;
+        for (int e = 0; e < n; ++e) {
+            // value plus float32 residual, as diag_weight adds them
+            const double hi = pool_entry(b, p.red_off, e).x;
+            B.f64(c128 ? hi : hi + pool_entry(b, p.red_off, n + e).x);
+        }
+    } else if (p.red_kind == RED_FORMS) {
+        if (p.red_k != 1 || p.red_R > 4) return false;
+        B.align(4);
+        B.w[RB_COEF] = (int)B.w.size();
+        for (int e = 0; e < 2 * 4 * p.red_R; ++e) {
+            const double2 v = pool_entry(b, p.red_off, e);
+            B.real(v.x);
+            B.real(v.y);
+        }
+    } else if (p.red_k > 4) {
+        return false;
+    }
+    const DecideDesc& d = *dec;
+    const bool j1 = d.kind == DEC_KRAUS_J1;
+    if (d.kind != DEC_KRAUS && d.kind != DEC_MEASURE && !j1) return false;
+    if (d.n_tail != (j1 ? 1 : 0) || (j1 && d.tail[0].kind != DEC_KRAUS_J2)) return false;
+    if (d.fork || d.sample_only || d.R * (j1 ? d.r2 : 1) != p.red_R) return false;
+    B.align(4);
+    int32_t D[RD_WORDS] = {};
+    D[RD_KIND] = d.kind;
+    D[RD_R] = d.R;
+    D[RD_PEND] = d.pend;
+    D[RD_OP] = (int32_t)d.op;
+    D[RD_R2] = j1 ? d.r2 : 1;
+    D[RD_OP2] = j1 ? (int32_t)d.tail[0].op : 0;
+    D[RD_PEND2] = j1 ? d.tail[0].pend : 0;
+    D[RD_M] = d.m;
+    for (int j = 0; j < d.m; ++j) D[RD_CLBITS] |= d.clbit[j] << (8 * j);  // at most 4
+    B.w[RB_DECIDE] = (int)B.w.size();
+    B.w.insert(B.w.end(), D, D + RD_WORDS);
+    B.align(4);
+    return true;
+}
+
+// A recorded pass as blocks.  A folded pass is one block on its qubits in
+// ascending order (the order of its groups' amplitudes).  Otherwise stages
+// join a block while its dense stages act on at most two qubits (a dense
+// two-qubit matrix fixes their order: its products are summed in column
+// order) and all of its stages on at most four; the reduction's block holds
+// the reduced qubits first, then the pass's other qubits in ascending order.
+bool res_pass(sv_batch b, const PassDesc& p, const DecideDesc* dec, int np, std::vector<std::vector<int32_t>>& out,
+              int* br_bytes) {
+    if (p.whole || (p.red_kind != RED_NONE) != (dec != nullptr)) return false;
+    // complex64 passes on shared-memory tiles round differently
+    if (b->prec == SV_C64 && p.reg_wp == 0) return false;
+    uint64_t act = 0;
+    for (int s = 0; s < p.n_stages; ++s)
+        for (int j = 0; j < p.st[s].k; ++j) act |= 1ull << p.tile_q[p.st[s].pos[j]];
+    std::vector<int> redq;
+    for (int j = 0; dec && j < p.red_k; ++j) {
+        redq.push_back(p.tile_q[p.red_pos[j]]);
+        act |= 1ull << redq.back();
+    }
+    if (__builtin_popcountll(act) > 4) return false;
+    std::vector<int> others;  // the pass's qubits without the reduced ones
+    for (int q = 0; q < np; ++q)
+        if (((act >> q) & 1) && std::find(redq.begin(), redq.end(), q) == redq.end()) others.push_back(q);
+    auto emit_block = [&](int s0, int s1, const std::vector<int>& fixed, const DecideDesc* d) {
+        ResBlock B;
+        int br = 0;
+        if (!res_block(b, p, s0, s1, fixed, d, np, B, &br)) return false;
+        *br_bytes = std::max(*br_bytes, br);
+        out.push_back(std::move(B.w));
+        return true;
+    };
+    if (p.fold) return !dec && emit_block(0, p.n_stages, others, nullptr);
+    std::vector<int> red_fixed = redq;
+    red_fixed.insert(red_fixed.end(), others.begin(), others.end());
+    auto add = [](std::vector<int>& v, int q) {
+        if (std::find(v.begin(), v.end(), q) == v.end()) v.push_back(q);
+    };
+    int s0 = 0;
+    std::vector<int> pair, extra;  // dense qubits, mask-stage qubits
+    bool ordered = false;          // a dense two-qubit matrix has fixed the pair's order
+    for (int s = 0; s < p.n_stages; ++s) {
+        const Stage& st = p.st[s];
+        const bool dense = st.kind == ST_DENSE || st.kind == ST_DENSE_BR;
+        if (dense && st.k > 2) return false;
+        std::vector<int> q;
+        for (int j = 0; j < st.k; ++j) q.push_back(p.tile_q[st.pos[j]]);
+        bool mono = false;  // every term monomial: either order
+        if (dense && st.k == 2 && !(st.kind == ST_DENSE_BR && st.pend == PEND_PSET)) {
+            auto it = b->term_count.find(st.off);
+            const int terms = st.kind == ST_DENSE ? 1 : (it == b->term_count.end() ? 0 : it->second);
+            mono = terms > 0;
+            for (int t = 0; t < terms && mono; ++t) {
+                double2 m[16], ph[4];
+                for (int e = 0; e < 16; ++e) m[e] = pool_entry(b, st.off + (int64_t)t * st.stride, e);
+                mono = mono_info(m, ph) != 0;
+            }
+        }
+        const bool fixes = dense && st.k == 2 && !mono;
+        std::vector<int> np_ = pair, ne = extra;
+        for (int x : q) add(dense ? np_ : ne, x);
+        std::vector<int> all = np_;
+        for (int x : ne) add(all, x);
+        bool fits_block = np_.size() <= 2 && all.size() <= 4;
+        if (fixes && fits_block) {
+            if (ordered) fits_block = np_[0] == q[0] && np_[1] == q[1];
+            else np_ = q;  // the same two qubits, in the matrix's order
+        }
+        if (!fits_block) {
+            std::vector<int> fixed = pair;
+            for (int x : extra) add(fixed, x);
+            if (!emit_block(s0, s, fixed, nullptr)) return false;
+            s0 = s;
+            pair.clear();
+            extra.clear();
+            ordered = false;
+            --s;
+            continue;
+        }
+        pair = np_;
+        extra = ne;
+        ordered = ordered || fixes;
+    }
+    std::vector<int> fixed = pair;
+    for (int x : extra) add(fixed, x);
+    if (!dec) return emit_block(s0, p.n_stages, fixed, nullptr);
+    // the last stages join the reduction when its qubit order suits them
+    bool joins = true;
+    for (size_t j = 0; j < pair.size(); ++j) {
+        const size_t at = std::find(red_fixed.begin(), red_fixed.end(), pair[j]) - red_fixed.begin();
+        joins = joins && (ordered ? at == j : at < 2);
+    }
+    if (!joins) {
+        if (!emit_block(s0, p.n_stages, fixed, nullptr)) return false;
+        s0 = p.n_stages;
+    }
+    return emit_block(s0, p.n_stages, red_fixed, dec);
+}
+
+// a recorded batch-mode circuit as one resident launch; false (and the
+// launches unchanged) when a pass, a decide or the sizes do not fit
+bool build_resident(sv_batch b, std::vector<Launch>& launches) {
+    const size_t ipool0 = b->ipool.size();
+    ResDesc r;
+    memset(&r, 0, sizeof(r));
+    r.np = std::max(4, b->n);
+    std::vector<std::vector<int32_t>> blocks;
+    int n_passes = 0;
+    bool ok = (int)b->pre_rows.size() <= RES_MAX_ROWS;
+    for (size_t i = 0; i < launches.size() && ok; ++i) {
+        const Launch& L = launches[i];
+        if (L.type == L_FINAL) {
+            ok = i + 1 == launches.size();
+            r.has_final = 1;
+            r.fin_op = L.fin.op;
+        } else if (L.type == L_PASS) {
+            ++n_passes;
+            const DecideDesc* dec = nullptr;
+            if (L.pass.red_kind != RED_NONE) {
+                if (i + 1 < launches.size() && launches[i + 1].type == L_DECIDE) dec = &launches[i + 1].dec;
+                ++i;
+            }
+            ok = res_pass(b, L.pass, dec, r.np, blocks, &r.br_bytes);
+        } else {
+            ok = false;
+        }
+    }
+    // batches: a reduction ends one (its choices are read by what follows)
+    r.mb = resident_batch(b->prec == SV_C128, r.np);
+    std::vector<int32_t> batches;
+    for (size_t i = 0; i < blocks.size(); ++i) {
+        const std::vector<int32_t>& w = blocks[i];
+        r.block_words = std::max(r.block_words, (int)w.size());
+        r.max_stages = std::max(r.max_stages, w[RB_NSTAGES]);
+        r.folds |= w[RB_FOLD];
+        const size_t n = batches.size();
+        if (n && batches[n - 1] < r.mb && blocks[i - 1][RB_RED] == RED_NONE) {
+            batches[n - 1] += 1;
+        } else {
+            batches.push_back((int32_t)i);
+            batches.push_back(1);
+        }
+    }
+    r.n_batches = (int)batches.size() / 2;
+    r.n_rows = (int)b->pre_rows.size();
+    if (!ok || resident_smem_bytes(b->prec == SV_C128, r) > RES_MAX_SMEM) {
+        b->ipool.resize(ipool0);
+        return false;
+    }
+    r.row_table = push_row_table(b);
+    std::vector<int32_t> index;
+    for (const std::vector<int32_t>& w : blocks) {
+        while (b->ipool.size() & 3) b->ipool.push_back(0);
+        index.push_back((int32_t)b->ipool.size());
+        index.push_back((int32_t)w.size());
+        b->ipool.insert(b->ipool.end(), w.begin(), w.end());
+    }
+    while (b->ipool.size() & 3) b->ipool.push_back(0);
+    r.index_off = (int)b->ipool.size();
+    b->ipool.insert(b->ipool.end(), index.begin(), index.end());
+    r.batch_off = (int)b->ipool.size();
+    b->ipool.insert(b->ipool.end(), batches.begin(), batches.end());
+    Launch L;
+    L.type = L_RESIDENT;
+    L.a0 = n_passes;
+    L.a1 = (int)b->n_shots;
+    L.res = r;
+    launches.assign(1, L);
+    return true;
+}
+
+// the circuit is one resident launch (which starts from |0...0> by itself)
+bool is_resident(const std::vector<Launch>& launches) { return launches.size() == 1 && launches[0].type == L_RESIDENT; }
+
+sv_status record_ops(sv_batch b, const sv_circuit* c, std::vector<Launch>& launches) {
     sv_status st = reset_pool(b);
     if (st) return st;
     b->pool_gen += 1;
@@ -1637,6 +2094,9 @@ sv_status record_circuit(sv_batch b, const sv_circuit* c, std::vector<Launch>& l
     b->rec = &launches;
     b->col_used = 0;
     b->pre_rows.clear();
+    b->term_count.clear();
+    b->term_count_i.clear();
+    launches.clear();
     for (int i = 0; i < c->n_ops && !st; ++i) {
         if (b->joint && i + 1 < c->n_ops && c->kind[i] == SV_OP_KRAUS && c->kind[i + 1] == SV_OP_KRAUS &&
             c->nq[i] == 1 && c->nq[i + 1] == 1 && c->qubits[c->q_off[i]] != c->qubits[c->q_off[i + 1]] &&
@@ -1651,8 +2111,21 @@ sv_status record_circuit(sv_batch b, const sv_circuit* c, std::vector<Launch>& l
     }
     if (!st) st = flush(b);
     b->rec = nullptr;
-    if (!st && !b->pre_rows.empty()) st = finish_predraw(b, launches);
+    return st;
+}
+
+sv_status record_circuit(sv_batch b, const sv_circuit* c, std::vector<Launch>& launches) {
+    sv_status st;
+    b->rec_resident = resident_candidate(b);
+    st = record_ops(b, c, launches);
+    const bool candidate = b->rec_resident;
+    b->rec_resident = false;
     if (st) return st;
+    if (candidate) {
+        if (build_resident(b, launches)) return upload_pool(b);
+        if ((uint64_t)b->pre_rows.size() * b->n_shots > PRE_TABLE_BYTES && (st = record_ops(b, c, launches))) return st;
+    }
+    if (!b->pre_rows.empty() && (st = finish_predraw(b, launches))) return st;
     return upload_pool(b);
 }
 
@@ -1810,7 +2283,7 @@ sv_status sv_alloc_batch(int n_qubits, uint64_t n_shots, int n_clbits, sv_prec p
     d.pool = b->d_pool;
     d.ipool = b->d_ipool;
     d.pass_log_cap = 1 << 20;
-    if (init_kernels() != cudaSuccess) {
+    if (init_kernels() != cudaSuccess || init_resident() != cudaSuccess) {
         sv_free_batch(b);
         return fail(SV_ECUDA, "cannot configure the kernels");
     }
@@ -1854,6 +2327,17 @@ sv_status sv_set_option(sv_batch b, sv_option opt, int64_t v) {
     // options shape the recorded launches (and the device struct the
     // kernels take by value): a cached graph is recorded again
     if (st == SV_OK && opt != SV_OPT_UPLOAD && opt != SV_OPT_PROFILE) b->pool_gen += 1;
+    if (st == SV_OK) {
+        bool off_default = false;  // an option that shapes passes, away from its default
+        switch (opt) {
+        case SV_OPT_TILE_BITS: case SV_OPT_MAX_ACTIVE: case SV_OPT_MAX_STAGES: case SV_OPT_THREADS:
+        case SV_OPT_GRID: case SV_OPT_PASS_PATH: case SV_OPT_WHOLE_STATE: off_default = v != 0; break;
+        case SV_OPT_JOINT_KRAUS: case SV_OPT_CHAIN_DECIDES: case SV_OPT_PREDRAW_PAULI: case SV_OPT_COMMUTE:
+        case SV_OPT_FOLD: off_default = v == 0; break;
+        default: break;
+        }
+        b->tuned = off_default ? b->tuned | 1u << opt : b->tuned & ~(1u << opt);
+    }
     return st;
 }
 
@@ -2060,9 +2544,18 @@ sv_status sv_run_circuit(sv_batch b, const sv_circuit* c, int use_graph) {
     }
     // launch list of the op sequence (after the reset / init of the root)
     const uint64_t h = circuit_hash(b, c);
-    const bool cached = use_graph && b->graph_exec && b->graph_hash == h && b->graph_gen == b->pool_gen;
+    // a resident circuit is one launch: kept as it is, no graph
+    const bool res_cached = use_graph && !b->res_list.empty() && b->res_hash == h && b->res_gen == b->pool_gen;
+    const bool cached = res_cached || (use_graph && b->graph_exec && b->graph_hash == h && b->graph_gen == b->pool_gen);
     std::vector<Launch> launches;
-    if (!cached && (st = record_circuit(b, c, launches))) return st;
+    if (res_cached) launches = b->res_list;
+    else if (!cached && (st = record_circuit(b, c, launches))) return st;
+    const bool resident = is_resident(launches);
+    if (resident && use_graph && !cached) {
+        b->res_list = launches;
+        b->res_hash = h;
+        b->res_gen = b->pool_gen;
+    }
     if (cached && b->upload_each) {
         // the circuit's constants cross the bus again (end-to-end timing)
         b->pool_up = 0;
@@ -2082,9 +2575,9 @@ sv_status sv_run_circuit(sv_batch b, const sv_circuit* c, int use_graph) {
         if ((st = exec(b, r))) return st;
         Launch in;
         in.type = L_INIT;
-        in.a0 = root_slots(b, n_run);
+        in.a0 = resident ? 0 : root_slots(b, n_run);
         if ((st = exec(b, in))) return st;
-        if (use_graph) {
+        if (use_graph && !resident) {
             if (!cached && round == 0) {
                 if (b->graph_exec) {
                     cudaGraphExecDestroy(b->graph_exec);
@@ -2105,7 +2598,7 @@ sv_status sv_run_circuit(sv_batch b, const sv_circuit* c, int use_graph) {
                 b->graph_hash = h;
                 b->graph_gen = b->pool_gen;
                 int64_t nl = 0;
-                for (const Launch& L : launches) nl += L.type == L_FINAL ? 3 : (L.type == L_DECIDE ? 2 : 1);
+                for (const Launch& L : launches) nl += launch_kernels(L);
                 b->graph_launches = nl;
                 b->graph_pass_store.clear();
                 for (const Launch& L : launches)
@@ -2185,13 +2678,7 @@ static sv_status capture_branches(sv_batch* bs, const std::vector<std::vector<La
 }
 
 static void count_launches(sv_batch b, const std::vector<Launch>& list) {
-    for (const Launch& L : list) {
-        b->n_launch += L.type == L_FINAL ? 3 : (L.type == L_DECIDE ? 2 : 1);
-        if (L.type == L_PASS) {
-            b->n_passes += 1;
-            b->pass_store.push_back(L.pass.store ? 1 : 0);
-        }
-    }
+    for (const Launch& L : list) count_launch(b, L);
 }
 
 sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int use_graph) {
@@ -2219,6 +2706,8 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
         b0->multi_lists.assign(n, {});
         for (int i = 0; i < n; ++i) {
             std::vector<Launch>& L = b0->multi_lists[i];
+            std::vector<Launch> ops;
+            if ((st = record_circuit(bs[i], cs[i], ops))) return st;
             Launch r;
             r.type = L_RESET;
             r.a0 = bs[i]->branch;
@@ -2227,10 +2716,8 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
             L.push_back(r);
             Launch in;
             in.type = L_INIT;
-            in.a0 = root_slots(bs[i], (int)bs[i]->n_shots);
+            in.a0 = is_resident(ops) ? 0 : root_slots(bs[i], (int)bs[i]->n_shots);
             L.push_back(in);
-            std::vector<Launch> ops;
-            if ((st = record_circuit(bs[i], cs[i], ops))) return st;
             L.insert(L.end(), ops.begin(), ops.end());
         }
     }
@@ -2599,7 +3086,8 @@ sv_status sv_stats(sv_batch b, double* s) {
     const int np = std::min<int>(ctl[CTL_NPASS], b->dev.pass_log_cap);
     std::vector<int32_t> nbr(np);
     if (np) CU(cudaMemcpy(nbr.data(), b->dev.pass_log, 4 * np, cudaMemcpyDeviceToHost));
-    double bytes = 0;
+    double bytes = b->res_bytes;
+    b->res_bytes = 0;
     for (int i = 0; i < np && i < (int)b->pass_store.size(); ++i)
         bytes += (double)nbr[i] * (double)b->state_bytes * (1.0 + b->pass_store[i]);
     s[0] = ctl[CTL_NBR];
