@@ -1239,14 +1239,13 @@ __global__ void __launch_bounds__(256) k_final_partials(DevBatch d, FinalDesc f)
     __shared__ double red_sh[32];
     const int n_br = d.ctl[CTL_NBR];
     const int64_t L = d.dim / f.chunks;
-    const int64_t items = (int64_t)n_br * f.chunks;
-    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
-        const int b = (int)(it / f.chunks), c = (int)(it % f.chunks);
-        const int slot = d.br_slot[b];
-        const T* g = reinterpret_cast<const T*>(d.states) + (int64_t)slot * d.dim + c * L;
-        const double s = svs::chunk_sum<R>(g, L, red_sh);
-        if (threadIdx.x == 0) d.partials[((int64_t)slot * d.max_chunks + c) * MAX_RED] = s;
-    }
+    svs::chunk_sums<R>(
+        (int64_t)n_br * f.chunks, f.chunks, L, red_sh,
+        [&](int64_t b) { return reinterpret_cast<const T*>(d.states) + (int64_t)d.br_slot[b] * d.dim; },
+        [&](int64_t it, double s) {
+            const int slot = d.br_slot[it / f.chunks];
+            d.partials[((int64_t)slot * d.max_chunks + it % f.chunks) * MAX_RED] = s;
+        });
 }
 
 // per branch (one warp): running sum of the chunk sums (into partials[..][1])

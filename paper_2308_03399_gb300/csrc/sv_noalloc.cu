@@ -42,15 +42,11 @@ __global__ void __launch_bounds__(256) na_partials(const typename svs::Cx<R>::T*
                                                   int n_states, double* scratch) {
     __shared__ double red_sh[32];
     const int64_t L = dim / chunks;
-    const int64_t items = (int64_t)n_states * chunks;
-    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
-        const int st = (int)(it / chunks), c = (int)(it % chunks);
-        const double s = svs::chunk_sum<R>(states + (int64_t)st * dim + c * L, L, red_sh);
-        if (threadIdx.x == 0) scratch[(int64_t)st * chunks + c] = s;
-    }
+    svs::chunk_sums<R>(
+        (int64_t)n_states * chunks, chunks, L, red_sh, [&](int64_t st) { return states + st * dim; },
+        [&](int64_t it, double s) { scratch[it] = s; });
 }
 
-// per state (one warp): running sum of its chunk sums, in place
 __global__ void __launch_bounds__(256) na_cum(int chunks, int n_states, double* scratch) {
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     for (int st = gw; st < n_states; st += nw)
@@ -124,7 +120,9 @@ extern "C" sv_status sv_final_sample_noalloc(const void* states, sv_prec prec, i
     }
     int n_sm = 0;
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = 2 * (n_sm > 0 ? n_sm : 1);
+    // HBM-bound: a full SM of warps (eight CTAs).  With two CTAs a SM the sums
+    // of 3001 states of 15 qubits took 450 us a call (1.75 TB/s).
+    const int grid = 8 * (n_sm > 0 ? n_sm : 1);
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     if (prec == SV_C128) {
         const double2* st = static_cast<const double2*>(states);

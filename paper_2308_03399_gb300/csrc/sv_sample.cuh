@@ -4,8 +4,9 @@
 // (sv_noalloc.cu), so both give the same key for the same state and draw.
 //
 // A state of 2^n amplitudes is cut into `chunks` contiguous chunks of L
-// amplitudes.  chunk_sum() gives one chunk's sum of |psi_j|^2 (one CTA,
-// float-float or float64 per thread, fixed-order combination); chunk_cum()
+// amplitudes.  chunk_sum() / chunk_sum_warp() give one chunk's sum of
+// |psi_j|^2 (one CTA or one warp, float-float or float64 per lane, fixed-order
+// combination); chunk_cum()
 // turns a state's chunk sums into a running sum (one warp, fixed order);
 // sample_warp() draws one key: the chunk by a two-level warp search over the
 // running sums, then the first j with u < C_j by a warp prefix sum over 256
@@ -53,6 +54,7 @@ template <class R> struct Sum;
 template <> struct Sum<double> {
     double s = 0.0;
     __device__ __forceinline__ void add_sq(double x, double y) { s += x * x + y * y; }
+    __device__ __forceinline__ void merge_xor(int o) { s += __shfl_xor_sync(0xffffffffu, s, o); }
     __device__ __forceinline__ double get() const { return s; }
 };
 // float-float pair (Knuth's TwoSum); the squares of float32 values enter
@@ -73,27 +75,86 @@ template <> struct Sum<float> {
         add(py);
         lo = __fadd_rn(lo, __fadd_rn(ex, ey));
     }
+    // plus the pair of lane ^ o (TwoSum of the high words, renormalised)
+    __device__ __forceinline__ void merge_xor(int o) {
+        const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float s = __fadd_rn(hi, bh);
+        const float bp = __fsub_rn(s, hi);
+        float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(bh, bp));
+        e = __fadd_rn(e, __fadd_rn(lo, bl));
+        hi = __fadd_rn(s, e);
+        lo = __fsub_rn(e, __fsub_rn(hi, s));
+    }
     __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
 };
+
+// the warp's sum (every lane; fixed order).  float-float pairs meet on the
+// float32 pipe: float64 adds retire two lanes per clock per SM, and a tree of
+// them for every 16 KB of amplitudes costs more than reading them
+template <class R> __device__ __forceinline__ double warp_sum_of(Sum<R> a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a.merge_xor(o);
+    return a.get();
+}
+
+// amplitudes j and j + 1 (j even): one 128-bit load where the state starts on
+// a 16-byte boundary
+__device__ __forceinline__ void add_pair(Sum<float>& a, float4 v) {
+    a.add_sq(v.x, v.y);
+    a.add_sq(v.z, v.w);
+}
+__device__ __forceinline__ float4 load_pair(const float2* g, bool aligned) {
+    if (aligned) return *reinterpret_cast<const float4*>(g);
+    const float2 x = g[0], y = g[1];
+    return make_float4(x.x, x.y, y.x, y.y);
+}
+
+// lanes first, first + step, ... (in units of two amplitudes for complex64,
+// one for complex128) of g[0..L): eight loads in flight
+template <class R>
+__device__ __forceinline__ void sum_strided(Sum<R>& a, const typename Cx<R>::T* g, int64_t L, int first, int step) {
+    if constexpr (sizeof(R) == 4) {
+        const bool aligned = (reinterpret_cast<uintptr_t>(g) & 15) == 0;
+        const int64_t n = L / 2;  // L is a power of two, at least 2
+        for (int64_t j0 = first; j0 < n; j0 += 8 * (int64_t)step) {
+            float4 v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (j0 + k * (int64_t)step < n) v[k] = load_pair(g + 2 * (j0 + k * (int64_t)step), aligned);
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (j0 + k * (int64_t)step < n) add_pair(a, v[k]);
+        }
+    } else {
+        for (int64_t j0 = first; j0 < L; j0 += 8 * (int64_t)step) {
+            double2 v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (j0 + k * (int64_t)step < L) v[k] = g[j0 + k * (int64_t)step];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (j0 + k * (int64_t)step < L) a.add_sq(v[k].x, v[k].y);
+        }
+    }
+}
+
+// sum of |psi_j|^2 over g[0..L), one warp, every lane
+template <class R> __device__ __forceinline__ double chunk_sum_warp(const typename Cx<R>::T* g, int64_t L) {
+    Sum<R> a;
+    sum_strided<R>(a, g, L, threadIdx.x & 31, 32);
+    return warp_sum_of<R>(a);
+}
+
+// chunks of at most this many amplitudes take a warp each (no block barrier,
+// several chunks of a CTA in flight), longer ones a CTA
+constexpr int64_t WARP_CHUNK = 4096;
 
 // sum of |psi_j|^2 over g[0..L), whole CTA; result valid in thread 0
 template <class R>
 __device__ __forceinline__ double chunk_sum(const typename Cx<R>::T* g, int64_t L, double* sh32) {
     Sum<R> a;
-    // a thread adds j = tid, tid + blockDim, ... in increasing order; the
-    // loads of eight consecutive terms are issued before their adds
-    const int64_t bd = blockDim.x;
-    for (int64_t j0 = threadIdx.x; j0 < L; j0 += 8 * bd) {
-        typename Cx<R>::T v[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (j0 + k * bd < L) v[k] = g[j0 + k * bd];
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (j0 + k * bd < L) a.add_sq(v[k].x, v[k].y);
-    }
-    double x = a.get();
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    sum_strided<R>(a, g, L, threadIdx.x, blockDim.x);
+    const double x = warp_sum_of<R>(a);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) sh32[threadIdx.x >> 5] = x;
     __syncthreads();
@@ -101,6 +162,24 @@ __device__ __forceinline__ double chunk_sum(const typename Cx<R>::T* g, int64_t 
     if (threadIdx.x == 0)
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh32[w];
     return s;
+}
+
+// every chunk sum of n_states states (item = state x chunk): put(item, sum)
+// is called by one thread per item
+template <class R, class State, class Put>
+__device__ __forceinline__ void chunk_sums(int64_t items, int chunks, int64_t L, double* sh32, State state, Put put) {
+    if (L <= WARP_CHUNK) {
+        const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+        for (int64_t it = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < items; it += nw) {
+            const double s = chunk_sum_warp<R>(state(it / chunks) + (it % chunks) * L, L);
+            if ((threadIdx.x & 31) == 0) put(it, s);
+        }
+    } else {
+        for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+            const double s = chunk_sum<R>(state(it / chunks) + (it % chunks) * L, L, sh32);
+            if (threadIdx.x == 0) put(it, s);
+        }
+    }
 }
 
 // running sum of sums[0..chunks) (stride `stride` doubles) into cum (same
@@ -156,6 +235,19 @@ __device__ __forceinline__ int64_t sample_warp(const typename Cx<R>::T* g, int64
         double acc = c ? cum[(int64_t)(c - 1) * stride] : 0.0;
         const int64_t j0 = (int64_t)c * L;
         for (int64_t blk = 0; blk < L && key < 0; blk += 256) {
+            if constexpr (sizeof(R) == 4) {
+                // the block's total on the float32 pipe; the float64 prefix
+                // below only for the block that holds the draw
+                if (L > 256) {
+                    Sum<R> t;
+                    sum_strided<R>(t, g + j0 + blk, 256, lane, 32);
+                    const double tot = warp_sum_of<R>(t);
+                    if (!(u < acc + tot) && blk + 256 < L) {
+                        acc += tot;
+                        continue;
+                    }
+                }
+            }
             double pe[8];
             double tot = 0.0;
 #pragma unroll
