@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libsv.so")
 SOURCES = ["sv_kernels.cu", "sv_reg_c64.cu", "sv_reg_c64x.cu", "sv_reg_c128.cu", "sv_runtime.cu", "sv_noalloc.cu",
-           "sv_resident.cu", "sv_resident_c128.cu",
+           "sv_resident.cu", "sv_resident_c64.cu", "sv_resident_c128.cu",
            "sv_mlp.cu", "sv_dm.cu"]
 HEADERS = ["sv_internal.h", "sv_sample.cuh", os.path.join("..", "..", "include", "sv.h"), "sv_common.cuh", "sv_pass_reg.cuh", "sv_pass_whole.cuh",
            "sv_resident.cuh", "sv_resident.h"]

@@ -1,10 +1,11 @@
-// complex64 instantiations of the resident run and its launcher (the
-// complex128 ones are in sv_resident_c128.cu, so that the two compile in
-// parallel).
+// Launcher of the resident runs and the complex64 instantiations for circuits
+// with folded passes (the others are in sv_resident_c64.cu and
+// sv_resident_c128.cu, so that they compile in parallel).
 #include "sv_resident.cuh"
 
 namespace sv {
 
+const void* resident_kernel_c64(int threads);  // no folded passes
 const void* resident_kernel_c128(int threads);
 
 namespace {
@@ -16,9 +17,10 @@ template <class R> size_t res_smem(const ResDesc& p) {
            warps * MAX_RED * 8 + RES_MAX_FINAL_CHUNKS * 8 + MAX_PEND * 4 + (((size_t)p.n_rows + 15) & ~(size_t)15);
 }
 
-const void* res_fn(int prec, int threads) {
+const void* res_fn(int prec, int folds, int threads) {
     if (prec) return resident_kernel_c128(threads);
-    return threads > 128 ? (const void*)k_resident<float, 512> : (const void*)k_resident<float, 128>;
+    if (!folds) return resident_kernel_c64(threads);
+    return threads > 128 ? (const void*)k_resident<float, 512, true> : (const void*)k_resident<float, 128, true>;
 }
 
 }  // namespace
@@ -42,8 +44,8 @@ cudaError_t init_resident() {
     cudaError_t e = cudaSuccess;
     for (int prec = 0; prec < 2; ++prec)
         for (int t : {128, 512})
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(res_fn(prec, t), cudaFuncAttributeMaxDynamicSharedMemorySize,
+            for (int folds = 0; folds < 2 && e == cudaSuccess; ++folds)
+                e = cudaFuncSetAttribute(res_fn(prec, folds, t), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)RES_MAX_SMEM);
     return e;
 }
@@ -51,7 +53,7 @@ cudaError_t init_resident() {
 cudaError_t launch_resident(const DevBatch& d, int prec, const ResDesc& p, int n_states, int n_sm, cudaStream_t s) {
     const int threads = resident_threads(prec, p.np);
     const size_t smem = resident_smem_bytes(prec, p);
-    const void* f = res_fn(prec, threads);
+    const void* f = res_fn(prec, p.folds, threads);
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem);
     if (e != cudaSuccess) return e;

@@ -42,12 +42,15 @@ namespace sv {
 
 namespace {
 
-// CTA shapes: registers for 20 complex64 or 12 complex128 warps per SM
-template <class R, int NT> struct ResCta;
-template <> struct ResCta<float, 128> { static constexpr int min_blocks = 5; };
-template <> struct ResCta<float, 512> { static constexpr int min_blocks = 1; };
-template <> struct ResCta<double, 128> { static constexpr int min_blocks = 3; };
-template <> struct ResCta<double, 256> { static constexpr int min_blocks = 1; };
+// CTA shapes: CTAs of 128 threads per SM (registers), by precision and
+// whether the circuit has folded blocks.  A spilled word costs more than the
+// warps it buys: the state takes most of the SM's memory and leaves little
+// L1 behind it (a Kraus circuit of 12 qubits ran 18.6 ms at 12 warps a SM and
+// 22 ms at 20 with 300 bytes of spills).
+template <class R, int NT, bool FOLDS> struct ResCta { static constexpr int min_blocks = 1; };
+template <> struct ResCta<float, 128, true> { static constexpr int min_blocks = 4; };
+template <> struct ResCta<float, 128, false> { static constexpr int min_blocks = 4; };
+template <> struct ResCta<double, 128, false> { static constexpr int min_blocks = 2; };
 
 // Shared-memory index of amplitude a: the high bits are folded into the low
 // four, so that 16 lanes whose group indices differ in four address bits of
@@ -177,18 +180,29 @@ static __device__ __noinline__ void res_compose(const int4* act, int cnt, const 
         const int j0 = a.w & 15, j1 = (a.w >> 4) & 15;
         const float2* m = reinterpret_cast<const float2*>(smem + a.y);
         if (a.x == RA_ONE || a.x == RA_ONE_SHAPED) {
+            // every load before the first store: the compiler cannot move a
+            // load of one pair above the stores of another
             const float2 m0 = m[0], m1 = m[1], m2 = m[2], m3 = m[3];
+            float2 u[4], w[4];
+            int r0[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const int g = 4 * h + i, r0 = ((g >> j0) << (j0 + 1)) | (g & ((1 << j0) - 1)), r1 = r0 | (1 << j0);
-                const float2 u = col[fold_at(r0)], w = col[fold_at(r1)];
+                const int g = 4 * h + i, r = ((g >> j0) << (j0 + 1)) | (g & ((1 << j0) - 1));
+                r0[i] = fold_at(r);
+                u[i] = col[r0[i]];
+                w[i] = col[fold_at(r | (1 << j0))];
+            }
+            const int step = fold_at(1 << j0);
+            const bool diag = (a.z & 3) == 1;
+            const float2 p = diag ? m0 : m1, q = diag ? m3 : m2;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
                 float2 x, y;
                 if (a.x == RA_ONE) {
-                    x = row2(m0, m1, u, w);
-                    y = row2(m2, m3, u, w);
+                    x = row2(m0, m1, u[i], w[i]);
+                    y = row2(m2, m3, u[i], w[i]);
                 } else {
-                    const bool diag = (a.z & 3) == 1;
-                    const float2 p = diag ? m0 : m1, q = diag ? m3 : m2, pu = diag ? u : w, qu = diag ? w : u;
+                    const float2 pu = diag ? u[i] : w[i], qu = diag ? w[i] : u[i];
                     if (a.z & 4) {
                         x = make_float2(p.x * pu.x, p.x * pu.y);
                         y = make_float2(q.x * qu.x, q.x * qu.y);
@@ -197,33 +211,33 @@ static __device__ __noinline__ void res_compose(const int4* act, int cnt, const 
                         y = cmul_rn(q, qu);
                     }
                 }
-                col[fold_at(r0)] = x;
-                col[fold_at(r1)] = y;
+                col[r0[i]] = x;
+                col[r0[i] + step] = y;
             }
         } else if (a.x == RA_TWO || a.x == RA_MONO) {
             const int lo = j0 < j1 ? j0 : j1, hi = j0 < j1 ? j1 : j0;
+            const int s0 = fold_at(1 << j0), s1 = fold_at(1 << j1);
+            float2 v[2][4];
+            int at[2];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 int g = 2 * h + i;
                 g = ((g >> lo) << (lo + 1)) | (g & ((1 << lo) - 1));
                 g = ((g >> hi) << (hi + 1)) | (g & ((1 << hi) - 1));
-                const int r[4] = {g, g | (1 << j0), g | (1 << j1), g | (1 << j0) | (1 << j1)};
+                at[i] = fold_at(g);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int pq = a.x == RA_MONO ? (a.z >> (8 + 2 * q)) & 3 : q;
+                    v[i][q] = col[at[i] + (pq & 1 ? s0 : 0) + (pq & 2 ? s1 : 0)];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
                 float2 o[4];
                 if (a.x == RA_MONO) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int pq = (a.z >> (8 + 2 * q)) & 3;
-                        const float2 u = col[fold_at(g | ((pq & 1) << j0) | ((pq >> 1) << j1))];
-                        o[q] = a.z & 2 ? u : cmul_rn(m[q], u);
-                    }
+                    for (int q = 0; q < 4; ++q) o[q] = a.z & 2 ? v[i][q] : cmul_rn(m[q], v[i][q]);
                 } else {
-                    unsigned long long ap[4], as[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float2 u = col[fold_at(r[q])];
-                        ap[q] = pk2(u.x, u.y);
-                        as[q] = pk2(u.y, u.x);
-                    }
                     const ulonglong2* mx = reinterpret_cast<const ulonglong2*>(m);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
@@ -231,14 +245,14 @@ static __device__ __noinline__ void res_compose(const int4* act, int cnt, const 
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             const ulonglong2 mm = mx[q * 4 + e];
-                            acc = fma2(mm.x, ap[e], acc);
-                            acc = fma2(mm.y, as[e], acc);
+                            acc = fma2(mm.x, pk2(v[i][e].x, v[i][e].y), acc);
+                            acc = fma2(mm.y, pk2(v[i][e].y, v[i][e].x), acc);
                         }
                         o[q] = upk2(acc);
                     }
                 }
 #pragma unroll
-                for (int q = 0; q < 4; ++q) col[fold_at(r[q])] = o[q];
+                for (int q = 0; q < 4; ++q) col[at[i] + (q & 1 ? s0 : 0) + (q & 2 ? s1 : 0)] = o[q];
             }
         } else {  // Pauli string or projection: elementwise on rows, moved by a flip mask
             float2 o[8];
@@ -295,8 +309,69 @@ static __device__ __noinline__ int res_table(const float2* M, const int32_t* so,
     return K;
 }
 
-template <class R, int NT>
-__global__ void __launch_bounds__(NT, (ResCta<R, NT>::min_blocks)) k_resident(DevBatch d, const __grid_constant__ ResDesc p) {
+// a folded block on NG groups: out[r] = sum over the row's nonzero columns,
+// or over all columns, ascending
+template <int NG, class Off>
+__device__ __forceinline__ void res_sparse(float2* st, const float4* tab, int K, const int (&base)[NG], Off off) {
+    float2 o[NG][16];
+#pragma unroll
+    for (int j = 0; j < NG; ++j)
+#pragma unroll
+        for (int r = 0; r < 16; ++r) o[j][r] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int k = 0; k < K; ++k) {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const float4 m = tab[16 * k + r];
+#pragma unroll
+            for (int j = 0; j < NG; ++j) {
+                const float2 a = st[base[j] ^ __float_as_int(m.x)];
+                o[j][r].x = fmaf(m.y, a.x, fmaf(-m.z, a.y, o[j][r].x));
+                o[j][r].y = fmaf(m.y, a.y, fmaf(m.z, a.x, o[j][r].y));
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < NG; ++j)
+#pragma unroll
+        for (int r = 0; r < 16; ++r) st[base[j] ^ off(r)] = o[j][r];
+}
+
+template <int NG, class Off>
+__device__ __forceinline__ void res_dense(float2* st, const float4* M, const int (&base)[NG], Off off) {
+    float2 v[NG][16];
+#pragma unroll
+    for (int j = 0; j < NG; ++j)
+#pragma unroll
+        for (int r = 0; r < 16; ++r) v[j][r] = st[base[j] ^ off(r)];
+#pragma unroll 1
+    for (int r = 0; r < 16; r += 2) {
+        float2 x[NG], y[NG];
+#pragma unroll
+        for (int j = 0; j < NG; ++j) x[j] = y[j] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+            const float4 m = M[(r >> 1) * FOLD_LD + c];
+#pragma unroll
+            for (int j = 0; j < NG; ++j) {
+                const float2 a = v[j][c];
+                x[j].x = fmaf(m.x, a.x, fmaf(-m.y, a.y, x[j].x));
+                x[j].y = fmaf(m.x, a.y, fmaf(m.y, a.x, x[j].y));
+                y[j].x = fmaf(m.z, a.x, fmaf(-m.w, a.y, y[j].x));
+                y[j].y = fmaf(m.z, a.y, fmaf(m.w, a.x, y[j].y));
+            }
+        }
+        const int o0 = off(r), o1 = off(r + 1);
+#pragma unroll
+        for (int j = 0; j < NG; ++j) {
+            st[base[j] ^ o0] = x[j];
+            st[base[j] ^ o1] = y[j];
+        }
+    }
+}
+
+template <class R, int NT, bool FOLDS>
+__global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resident(DevBatch d, const __grid_constant__ ResDesc p) {
     using T = typename Cplx<R>::T;
     using A = typename AccSlot<R>::T;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -351,7 +426,9 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT>::min_blocks)) k_resident(De
             double scale = 1.0;
             int br_k = 0;
             if (s < n) {
-                const int32_t* S = B + RB_STAGES + RS_WORDS * s;
+                const int4 Sa = *reinterpret_cast<const int4*>(B + RB_STAGES + RS_WORDS * s);
+                const int4 Sb = *reinterpret_cast<const int4*>(B + RB_STAGES + RS_WORDS * s + 4);
+                const int S[7] = {Sa.x, Sa.y, Sa.z, Sa.w, Sb.x, Sb.y, Sb.z};
                 const int w0 = S[0], kind = w0 & 15, k = (w0 >> 4) & 15, pos = S[1];
                 on = true;
                 if ((w0 >> 10) & 1) on = (int)((clb >> ((w0 >> 12) & 63)) & 1) == ((w0 >> 11) & 1);
@@ -436,7 +513,7 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT>::min_blocks)) k_resident(De
             }
         }
         __syncwarp();
-        if constexpr (sizeof(T) == 8) {
+        if constexpr (FOLDS) {
             if (B[RB_FOLD]) {
                 if (count > 0) {
                     float2* M = reinterpret_cast<float2*>(works + q * 8 * FOLD_LD);
@@ -513,46 +590,24 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT>::min_blocks)) k_resident(De
             auto off = [&](int e) {
                 return ((e & 1) ? so0 : 0) ^ ((e & 2) ? so1 : 0) ^ ((e & 4) ? so2 : 0) ^ ((e & 8) ? so3 : 0);
             };
-            if (sizeof(T) == 8 && B[RB_FOLD]) {
-                if constexpr (sizeof(T) == 8) {
+            if (FOLDS && B[RB_FOLD]) {
+                if constexpr (FOLDS) {
                     const int K = n_act[q];
                     const float4* tab = tabs + q * 16 * FOLD_SPARSE;
                     const float4* M = works + q * 8 * FOLD_LD;
-                    for (int g = tid; K > 0 && g < groups; g += nth) {
-                        const int base = group_base(g);
-                        float2 o[16];
-                        if (K <= FOLD_SPARSE) {
-#pragma unroll
-                            for (int r = 0; r < 16; ++r) o[r] = make_float2(0.f, 0.f);
-                            for (int k = 0; k < K; ++k) {
-#pragma unroll
-                                for (int r = 0; r < 16; ++r) {
-                                    const float4 m = tab[16 * k + r];
-                                    const float2 a = st[base ^ __float_as_int(m.x)];
-                                    o[r].x = fmaf(m.y, a.x, fmaf(-m.z, a.y, o[r].x));
-                                    o[r].y = fmaf(m.y, a.y, fmaf(m.z, a.x, o[r].y));
-                                }
-                            }
-#pragma unroll
-                            for (int r = 0; r < 16; ++r) st[base ^ off(r)] = o[r];
+                    // A dense product is bound by delivering its matrix: a
+                    // 128-bit broadcast load returns 512 bytes to the warp,
+                    // four clocks of the SM, for eight FMAs.  Two groups per
+                    // thread share each load.
+                    for (int g = tid; K > 0 && g < groups; g += 2 * nth) {
+                        if (g + nth < groups) {
+                            const int base[2] = {group_base(g), group_base(g + nth)};
+                            if (K <= FOLD_SPARSE) res_sparse<2>(st, tab, K, base, off);
+                            else res_dense<2>(st, M, base, off);
                         } else {
-#pragma unroll
-                            for (int r = 0; r < 16; ++r) o[r] = st[base ^ off(r)];
-#pragma unroll 1
-                            for (int r = 0; r < 16; r += 2) {
-                                float2 x = make_float2(0.f, 0.f), y = make_float2(0.f, 0.f);
-#pragma unroll
-                                for (int c = 0; c < 16; ++c) {
-                                    const float4 m = M[(r >> 1) * FOLD_LD + c];
-                                    const float2 a = o[c];
-                                    x.x = fmaf(m.x, a.x, fmaf(-m.y, a.y, x.x));
-                                    x.y = fmaf(m.x, a.y, fmaf(m.y, a.x, x.y));
-                                    y.x = fmaf(m.z, a.x, fmaf(-m.w, a.y, y.x));
-                                    y.y = fmaf(m.z, a.y, fmaf(m.w, a.x, y.y));
-                                }
-                                st[base ^ off(r)] = x;
-                                st[base ^ off(r) ^ so0] = y;
-                            }
+                            const int base[1] = {group_base(g)};
+                            if (K <= FOLD_SPARSE) res_sparse<1>(st, tab, K, base, off);
+                            else res_dense<1>(st, M, base, off);
                         }
                     }
                 }
@@ -576,7 +631,16 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT>::min_blocks)) k_resident(De
                             if (r.w & 15) reg_apply1<T, 16, 1>(v, m);
                             else reg_apply1<T, 16, 0>(v, m);
                         } else if (r.x == RA_MONO) {
-                            reg_mono<T, 16, 0, 1>(v, r.z, m);
+                            if (r.z & RES_MONO_REAL) {  // real phases: half the products
+                                reg_mono<T, 16, 0, 1>(v, r.z | 2, m);
+#pragma unroll
+                                for (int e = 0; e < 16; ++e) {
+                                    v[e].x = m[e & 3].x * v[e].x;
+                                    v[e].y = m[e & 3].x * v[e].y;
+                                }
+                            } else {
+                                reg_mono<T, 16, 0, 1>(v, r.z, m);
+                            }
                         } else if (r.x == RA_TWO) {
                             if constexpr (sizeof(T) == 8)
                                 reg_apply2_f32x2<16, 0, 1>(reinterpret_cast<float2*>(v),
@@ -634,17 +698,15 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT>::min_blocks)) k_resident(De
                     // a warp owns an outcome: its amplitudes, one compensated
                     // addition each, in a fixed order
                     __syncthreads();
-                    const int rp = B[RB_RPOS];
+                    // (the measured qubits are group bits 0.. in order)
                     for (int o = warp; o < red_R; o += nw) {
                         Acc<R> a;
                         a.zero();
-                        for (int g = lane; g < groups; g += 32) {
-                            const int base = group_base(g);
-                            for (int e = 0; e < 16; ++e) {
-                                int b = 0;
-                                for (int j = 0; j < red_k; ++j) b |= ((e >> ((rp >> (4 * j)) & 15)) & 1) << j;
-                                if (b != o) continue;
-                                const T x = st[base ^ off(e)];
+                        for (int m = o; m < 16; m += red_R) {
+                            const int om = off(m);
+#pragma unroll 4
+                            for (int g = lane; g < groups; g += 32) {
+                                const T x = st[group_base(g) ^ om];
                                 a.add(x.x * x.x + x.y * x.y);
                             }
                         }

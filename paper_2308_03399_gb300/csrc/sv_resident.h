@@ -47,6 +47,8 @@ enum : int32_t {
 // entries of the active-stage list
 enum : int32_t { RA_ONE = 0, RA_ONE_SHAPED, RA_TWO, RA_MONO, RA_PAULI, RA_PROJ };
 
+constexpr int RES_MONO_REAL = 1 << 16;  // a monomial matrix's phases are real (with its mono_info)
+
 struct ResDesc {
     int32_t np;           // address bits of the state in shared memory (at least 4)
     int32_t n_batches;

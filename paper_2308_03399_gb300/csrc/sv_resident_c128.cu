@@ -4,7 +4,7 @@
 namespace sv {
 
 const void* resident_kernel_c128(int threads) {
-    return threads > 128 ? (const void*)k_resident<double, 256> : (const void*)k_resident<double, 128>;
+    return threads > 128 ? (const void*)k_resident<double, 256, false> : (const void*)k_resident<double, 128, false>;
 }
 
 }  // namespace sv

@@ -207,6 +207,11 @@ struct sv_batch_s {
     std::vector<Launch> res_list;
     uint64_t res_hash = 0, res_gen = 0;
     double res_bytes = 0;  // states written by resident runs since sv_stats
+    // resident runs of a shot-branching batch: a history word per shot, runs
+    // since sv_stats, and whether the last run was one
+    unsigned long long* d_hist = nullptr;
+    int64_t res_branch_runs = 0;
+    bool res_branch_last = false;
     std::map<int, int> term_count, term_count_i;  // terms at a pool / integer-pool offset (recording)
     // parameter sweep (sv_set_param_sets): every shot's parameter set
     int n_psets = 0;
@@ -318,6 +323,7 @@ void count_launch(sv_batch b, const Launch& L) {
         b->pass_store.push_back(L.pass.store ? 1 : 0);
     } else if (L.type == L_RESIDENT) {
         b->n_passes += L.a0;
+        b->res_branch_runs += b->branch;
         b->res_bytes += (double)L.a1 * (double)b->state_bytes;
     }
 }
@@ -1673,8 +1679,67 @@ sv_status finish_predraw(sv_batch b, std::vector<Launch>& launches) {
 constexpr int RES_MAX_QUBITS_C64 = 14, RES_MAX_QUBITS_C128 = 13;
 
 bool resident_candidate(sv_batch b) {
-    if (b->tuned || b->log || b->branch || b->mode == SV_PLAIN) return false;
+    if (b->tuned || b->log || b->mode == SV_PLAIN) return false;
+    // a state of its own for every shot (shot-branching with a slot each)
+    if ((uint64_t)b->dev.n_slots < b->n_shots) return false;
     return b->n <= (b->prec == SV_C128 ? RES_MAX_QUBITS_C128 : RES_MAX_QUBITS_C64);
+}
+
+// Shot-branching shares the states of shots that agree so far but pays a
+// decide, a copy and a pass launch per random op; a resident run simulates
+// every shot by itself in one launch.  Both are estimated in microseconds
+// from GB300 timings (circuits of 6 to 13 qubits, 100 to 4000 shots,
+// noise of 1e-4 to 3e-2): the
+// branching run from its launches and the number of live branches that the
+// noise probabilities lead to expect, the resident run from the passes of
+// every shot.  It has to come out clearly ahead.
+bool resident_pays(sv_batch b, const sv_circuit* c, const std::vector<Launch>& launches) {
+    const double S = (double)b->n_shots, dim = (double)b->dim;
+    const bool c128 = b->prec == SV_C128;
+    // expected live branches, averaged over the random ops; decides in chains
+    double keep = 1.0, live = 0.0, roots = std::max(1, b->n_psets);
+    int ops = 0, chains = 0, tail = 0;
+    for (int i = 0; i < c->n_ops; ++i) {
+        const int kind = c->kind[i], k = c->nq[i];
+        const double* d = c->data + c->d_off[i];
+        double p0 = 1.0;  // probability of the likeliest outcome
+        if (kind == SV_OP_PAULI) {
+            p0 = d[0];
+        } else if (kind == SV_OP_KRAUS) {
+            p0 = 0.0;
+            for (int t = 0; t < c->n_terms[i]; ++t) {
+                double w = 0.0;
+                for (int e = 0; e < 2 << (2 * k); ++e) w += d[(size_t)t * (2 << (2 * k)) + e] * d[(size_t)t * (2 << (2 * k)) + e];
+                p0 = std::max(p0, w / (1 << k));
+            }
+        } else if (kind == SV_OP_MEASURE) {
+            p0 = 1.0 / (1 << k);
+        } else {
+            if (kind == SV_OP_GATE && k > 2) tail = 0;
+            continue;
+        }
+        keep *= std::min(1.0, std::max(0.0, p0));
+        ++ops;
+        live += std::min(S, roots + S * (1.0 - keep));
+        // Pauli ops follow a decide as its tail, up to MAX_TAIL of them
+        if (kind == SV_OP_PAULI && tail < MAX_TAIL && ops > 1) ++tail;
+        else {
+            ++chains;
+            tail = 0;
+        }
+    }
+    if (ops) live /= ops;
+    double passes = 0;
+    for (const Launch& L : launches) {
+        if (L.type != L_PASS) continue;
+        passes += 1;
+    }
+    const double branch = chains * (14.0 + 0.0037 * S) + passes * (8.0 + std::min(dim, 8192.0) * (c128 ? 8e-3 : 4.3e-3)) +
+                          passes * live * (double)b->state_bytes * 2.0 / 3.5e6;
+    // per pass a latency floor, and nanoseconds of the chip per state
+    const double resident = c128 ? passes * std::max(12.0 + dim * 0.016, S * (35.0 + dim * 0.09) * 1e-3)
+                                 : passes * std::max(8.5, S * (6.0 + dim * 0.0026) * 1e-3);
+    return resident < 0.8 * branch;
 }
 
 // one block of a resident program: 32-bit words, matrices in the batch's
@@ -1812,6 +1877,8 @@ bool res_block(sv_batch b, const PassDesc& p, int s0, int s1, const std::vector<
                 }
                 info[t] = st.k == 1 ? shape1(m) : (pset ? 0 : mono_info(m, ph));
                 if (st.k == 2 && st.kind == ST_DENSE_BR) info[t] &= ~2;
+                if (st.k == 2 && info[t] && !(info[t] & 2) && ph[0].y == 0 && ph[1].y == 0 && ph[2].y == 0 && ph[3].y == 0)
+                    info[t] |= RES_MONO_REAL;
                 for (int j = 0; j < 4; ++j) phs[t][j] = ph[j];
                 all_mono = all_mono && info[t];
             }
@@ -2040,7 +2107,7 @@ bool build_resident(sv_batch b, std::vector<Launch>& launches) {
         }
     }
     // batches: a reduction ends one (its choices are read by what follows)
-    r.mb = resident_batch(b->prec == SV_C128, r.np);
+    const int most = resident_batch(b->prec == SV_C128, r.np);
     std::vector<int32_t> batches;
     for (size_t i = 0; i < blocks.size(); ++i) {
         const std::vector<int32_t>& w = blocks[i];
@@ -2048,18 +2115,27 @@ bool build_resident(sv_batch b, std::vector<Launch>& launches) {
         r.max_stages = std::max(r.max_stages, w[RB_NSTAGES]);
         r.folds |= w[RB_FOLD];
         const size_t n = batches.size();
-        if (n && batches[n - 1] < r.mb && blocks[i - 1][RB_RED] == RED_NONE) {
+        if (n && batches[n - 1] < most && blocks[i - 1][RB_RED] == RED_NONE) {
             batches[n - 1] += 1;
         } else {
             batches.push_back((int32_t)i);
             batches.push_back(1);
         }
+        r.mb = std::max(r.mb, batches.back());  // shared memory for the largest one
     }
+    r.mb = std::max(r.mb, 1);
     r.n_batches = (int)batches.size() / 2;
     r.n_rows = (int)b->pre_rows.size();
     if (!ok || resident_smem_bytes(b->prec == SV_C128, r) > RES_MAX_SMEM) {
         b->ipool.resize(ipool0);
         return false;
+    }
+    if (b->branch) {  // sv_stats counts the histories (see there)
+        if (!b->d_hist && dalloc(b, &b->d_hist, b->n_shots) != SV_OK) {
+            b->ipool.resize(ipool0);
+            return false;
+        }
+        r.hist = b->d_hist;
     }
     r.row_table = push_row_table(b);
     std::vector<int32_t> index;
@@ -2115,15 +2191,19 @@ sv_status record_ops(sv_batch b, const sv_circuit* c, std::vector<Launch>& launc
 }
 
 sv_status record_circuit(sv_batch b, const sv_circuit* c, std::vector<Launch>& launches) {
-    sv_status st;
-    b->rec_resident = resident_candidate(b);
-    st = record_ops(b, c, launches);
-    const bool candidate = b->rec_resident;
+    const bool candidate = resident_candidate(b), branch = b->branch;
+    b->rec_resident = candidate;
+    if (candidate) b->branch = false;  // every shot its own branch
+    sv_status st = record_ops(b, c, launches);
     b->rec_resident = false;
+    b->branch = branch;
     if (st) return st;
     if (candidate) {
-        if (build_resident(b, launches)) return upload_pool(b);
-        if ((uint64_t)b->pre_rows.size() * b->n_shots > PRE_TABLE_BYTES && (st = record_ops(b, c, launches))) return st;
+        if ((!branch || resident_pays(b, c, launches)) && build_resident(b, launches)) return upload_pool(b);
+        // the launches of the pass kernels instead
+        if ((branch || (uint64_t)b->pre_rows.size() * b->n_shots > PRE_TABLE_BYTES) &&
+            (st = record_ops(b, c, launches)))
+            return st;
     }
     if (!b->pre_rows.empty() && (st = finish_predraw(b, launches))) return st;
     return upload_pool(b);
@@ -2330,7 +2410,9 @@ sv_status sv_set_option(sv_batch b, sv_option opt, int64_t v) {
     if (st == SV_OK) {
         bool off_default = false;  // an option that shapes passes, away from its default
         switch (opt) {
-        case SV_OPT_TILE_BITS: case SV_OPT_MAX_ACTIVE: case SV_OPT_MAX_STAGES: case SV_OPT_THREADS:
+        // (a tile size that the state caps to the default one changes nothing)
+        case SV_OPT_TILE_BITS: off_default = b->tb != std::min(b->n, b->prec == SV_C128 ? 10 : 11); break;
+        case SV_OPT_MAX_ACTIVE: case SV_OPT_MAX_STAGES: case SV_OPT_THREADS:
         case SV_OPT_GRID: case SV_OPT_PASS_PATH: case SV_OPT_WHOLE_STATE: off_default = v != 0; break;
         case SV_OPT_JOINT_KRAUS: case SV_OPT_CHAIN_DECIDES: case SV_OPT_PREDRAW_PAULI: case SV_OPT_COMMUTE:
         case SV_OPT_FOLD: off_default = v == 0; break;
@@ -2562,7 +2644,8 @@ sv_status sv_run_circuit(sv_batch b, const sv_circuit* c, int use_graph) {
         b->ipool_up = 0;
         if ((st = upload_pool(b))) return st;
     }
-    const int branch = b->branch;
+    const int branch = b->branch && !resident;
+    b->res_branch_last = b->branch && resident;
     int from_wait = 0;
     int n_run = (int)b->n_shots;
     if ((st = tree_begin(b))) return st;
@@ -2710,7 +2793,7 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
             if ((st = record_circuit(bs[i], cs[i], ops))) return st;
             Launch r;
             r.type = L_RESET;
-            r.a0 = bs[i]->branch;
+            r.a0 = bs[i]->branch && !is_resident(ops);
             r.a1 = (int)bs[i]->n_shots;
             r.a2 = 0;
             L.push_back(r);
@@ -2721,6 +2804,13 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
             L.insert(L.end(), ops.begin(), ops.end());
         }
     }
+    // batches whose shots branch (a resident run leaves nothing waiting)
+    std::vector<char> forks(n, 0);
+    for (int i = 0; i < n; ++i) {
+        const bool resident = b0->multi_lists[i].back().type == L_RESIDENT;
+        forks[i] = bs[i]->branch && !resident;
+        bs[i]->res_branch_last = bs[i]->branch && resident;
+    }
     for (int i = 0; i < n; ++i)
         if ((st = tree_begin(bs[i]))) return st;
     if (!use_graph) {
@@ -2730,7 +2820,7 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
         // shot-branching batches whose forks found no slot: restart their
         // waiting lists one by one
         for (int i = 0; i < n; ++i) {
-            if (!bs[i]->branch) continue;
+            if (!forks[i]) continue;
             std::vector<Launch> ops(b0->multi_lists[i].begin() + 2, b0->multi_lists[i].end());
             if ((st = drain_waiting(bs[i], ops))) return st;
         }
@@ -2754,7 +2844,7 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
         std::vector<int> wait(n, 0);
         bool any = false;
         for (int i = 0; i < n; ++i) {
-            if (!bs[i]->branch) continue;
+            if (!forks[i]) continue;
             int32_t ctl[CTL_WORDS];
             if ((st = read_ctl(bs[i], ctl))) return st;
             if ((st = tree_snapshot(bs[i], ctl, (int)bs[i]->n_shots))) return st;
@@ -2766,7 +2856,7 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
             if (rl.empty())
                 for (int i = 0; i < n; ++i) {
                     std::vector<Launch> L;
-                    if (bs[i]->branch) {
+                    if (forks[i]) {
                         Launch r;
                         r.type = L_RESET;
                         r.a0 = 1;
@@ -2785,7 +2875,7 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
             CU(cudaGraphLaunch(b0->multi_restart_exec, b0->stream));
             any = false;
             for (int i = 0; i < n; ++i) {
-                if (!bs[i]->branch) continue;
+                if (!forks[i]) continue;
                 count_launches(bs[i], rl[i]);
                 if (wait[i] == 0) continue;
                 bs[i]->restarts += 1;
@@ -3090,12 +3180,30 @@ sv_status sv_stats(sv_batch b, double* s) {
     b->res_bytes = 0;
     for (int i = 0; i < np && i < (int)b->pass_store.size(); ++i)
         bytes += (double)nbr[i] * (double)b->state_bytes * (1.0 + b->pass_store[i]);
-    s[0] = ctl[CTL_NBR];
+    // a resident run of a shot-branching batch gave every shot a state of its
+    // own; the branches it stands for are the different histories
+    double live = ctl[CTL_NBR], copied = ctl[CTL_NCOPIED];
+    if (b->res_branch_last && b->d_hist) {
+        std::vector<unsigned long long> h(b->n_shots);
+        CU(cudaMemcpyAsync(h.data(), b->d_hist, 8 * b->n_shots, cudaMemcpyDeviceToHost, b->stream));
+        CU(cudaStreamSynchronize(b->stream));
+        std::sort(h.begin(), h.end());
+        live = (double)(std::unique(h.begin(), h.end()) - h.begin());
+        double roots = 1;
+        if (b->n_psets > 0) {
+            std::vector<uint32_t> ps(b->h_pset);
+            std::sort(ps.begin(), ps.end());
+            roots = (double)(std::unique(ps.begin(), ps.end()) - ps.begin());
+        }
+        copied += (double)b->res_branch_runs * (live - roots);
+    }
+    b->res_branch_runs = 0;
+    s[0] = live;
     s[1] = ctl[CTL_NWAIT];
     s[2] = (double)b->n_launch;
     s[3] = (double)b->n_passes;
     s[4] = bytes;
-    s[5] = (double)ctl[CTL_NCOPIED] * 2.0 * (double)b->state_bytes;
+    s[5] = copied * 2.0 * (double)b->state_bytes;
     s[6] = (double)b->restarts;
     s[7] = b->h2d_bytes;
     b->h2d_bytes = 0;
