@@ -244,7 +244,11 @@ sv_status sv_waiting(sv_batch b, uint64_t *n_waiting);
 /* Run a whole circuit for all shots (Sections IV-A and IV-B), restarting
  * the waiting list until it is empty, and leave per-shot keys for
  * sv_get_keys.  use_graph != 0 captures the launch sequence into a CUDA
- * graph once per circuit and replays it.                                    */
+ * graph once per circuit and replays it.  Small registers (up to 14 qubits,
+ * 13 in complex128) may run as one kernel with every shot's state in shared
+ * memory, in shot-branching modes too when each shot has a state slot; the
+ * results are the same.  SV_OPT_LOG, or a pass-shaping option away from its
+ * default, keeps a run on the pass kernels.                                 */
 sv_status sv_run_circuit(sv_batch b, const sv_circuit *c, int use_graph);
 
 /* Several circuits, one per batch (n of them, batches sharing one stream;

@@ -16,7 +16,11 @@ constexpr int64_t REG_UNIT_MIN_AMPS = 8192;  // smallest register-path unit
 constexpr int PRE_WORDS = 8;                 // integer-pool words per pre-drawn Pauli row
 constexpr uint64_t PRE_TABLE_BYTES = 1ull << 30;  // largest pre-drawn Pauli table
 constexpr int MAX_RED = 16;        // probabilities reduced by one pass (Kraus terms, 2^m outcomes)
-constexpr int MAX_CHUNKS = 1024;   // reduction partials per state
+// reduction partials per state: fine enough that the units of a few branches
+// of a large state still divide evenly over some 3000 warps (with 1024, three
+// 27-qubit branches left 98% of them idle in a second round: 4.2 TB/s)
+constexpr int MAX_CHUNKS = 8192;
+constexpr int MAX_FINAL_CHUNKS = 1024;  // chunks of the final sample
 constexpr int MAX_STAGE_Q = 5;     // qubits of one stage (dense gates up to MAX_GATE_Q)
 constexpr int MAT_SMEM = 1024;     // complex matrix entries staged in shared memory per pass
 // fork log record: op, parent branch, child branch (-1: waiting list), outcome,

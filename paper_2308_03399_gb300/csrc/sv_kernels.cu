@@ -617,8 +617,58 @@ struct DecTab {
 // probabilities of branch b into p_out (and, for Pauli, the table into
 // cum_out); one whole warp.  With joint_out (a DEC_KRAUS_J1 head), the
 // joint probabilities p_ij are kept there too.
+// where the terms of branch b's decide lie: the contiguous entries
+// [base, base + nk) of every chunk's record
+struct PartSrc {
+    const double* pp;
+    int nk, inner;
+};
+__device__ __forceinline__ PartSrc part_src(const DevBatch& d, const DecideDesc& dd, int b, int slot) {
+    int src = slot, base_r = 0, inner = 1;
+    if (dd.kind == DEC_KRAUS_J1) {
+        inner = dd.r2;  // p_i = sum over j of the joint p_ij = entry i * r2 + j
+    } else if (dd.kind == DEC_KRAUS_J2) {
+        // branches forked by the first op still find the joint partials in
+        // their parent's slot
+        const int cf = d.ctl[CTL_COPY_FIRST], ce = d.ctl[CTL_COPY_END];
+        if (b >= cf && b < ce) src = d.br_slot[d.br_parent[b]];
+        base_r = d.br_sel[(int64_t)dd.pend_prev * d.cap_br + b] * dd.R;  // p_ij = entry i * R + j
+    }
+    return {d.partials + (int64_t)src * d.max_chunks * MAX_RED + base_r, dd.R * inner, inner};
+}
+
+// this warp's share (chunks w, w + nw, ... in blocks of 32) of the sums of a
+// branch's terms, into out[0..nk) (lane 0)
+__device__ __forceinline__ void part_sums(const PartSrc& ps, int chunks, int w, int nw, double* out) {
+    const int lane = threadIdx.x & 31;
+    double u[MAX_RED];
+#pragma unroll
+    for (int k = 0; k < MAX_RED; ++k) u[k] = 0.0;
+    for (int c = 32 * w + lane; c < chunks; c += 32 * nw) {
+        const double* q = ps.pp + (int64_t)c * MAX_RED;
+#pragma unroll
+        for (int k = 0; k < MAX_RED; ++k)
+            if (k < ps.nk) u[k] += q[k];
+    }
+#pragma unroll
+    for (int k = 0; k < MAX_RED; ++k)
+        if (k < ps.nk) {
+            const double t = warp_sum(u[k], chunks - 32 * w < 0 ? 0 : chunks - 32 * w);
+            if (lane == 0) out[k] = t;
+        }
+}
+
+// Branches whose sums run over more chunks than this take a CTA whatever
+// their shots: a warp adding the 8192 chunks of a 27-qubit state needs
+// longer than a small state's whole pass
+constexpr int DEC_WARP_CHUNKS = 512;
+__device__ __forceinline__ bool decide_in_cta(const DecideDesc& dd, int cnt) {
+    return cnt > DEC_SMALL || (dd.kind != DEC_PAULI && dd.chunks > DEC_WARP_CHUNKS);
+}
+
+// pre: per warp of the CTA its share of the sums (part_sums), nullable
 __device__ void warp_probs(const DevBatch& d, const DecideDesc& dd, int b, int slot, double* p_out, double* cum_out,
-                           double* joint_out) {
+                           double* joint_out, const double (*pre)[MAX_RED], int npre) {
     const int lane = threadIdx.x & 31;
     const int R = dd.R;
     if (dd.kind == DEC_PAULI) {
@@ -629,38 +679,21 @@ __device__ void warp_probs(const DevBatch& d, const DecideDesc& dd, int b, int s
         __syncwarp();
         return;
     }
-    // The terms needed are the contiguous entries [base_r, base_r + R*inner)
-    // of every chunk's record: p_r = sum over chunks and j < inner of
-    // entry base_r + r*inner + j.  Each lane adds its chunks' entries in
-    // registers (all loads of a chunk issued together), the lanes' sums are
-    // combined by the fixed shuffle tree, and lane 0 adds the inner terms.
-    int src = slot, base_r = 0, inner = 1;
-    if (dd.kind == DEC_KRAUS_J1) {
-        inner = dd.r2;  // p_i = sum over j of the joint p_ij = entry i * r2 + j
-    } else if (dd.kind == DEC_KRAUS_J2) {
-        // branches forked by the first op still find the joint partials in
-        // their parent's slot
-        const int cf = d.ctl[CTL_COPY_FIRST], ce = d.ctl[CTL_COPY_END];
-        if (b >= cf && b < ce) src = d.br_slot[d.br_parent[b]];
-        base_r = d.br_sel[(int64_t)dd.pend_prev * d.cap_br + b] * R;  // p_ij = entry i * R + j
-    }
-    const int nk = R * inner;
-    const double* pp = d.partials + (int64_t)src * d.max_chunks * MAX_RED + base_r;
-    double u[MAX_RED];
-#pragma unroll
-    for (int k = 0; k < MAX_RED; ++k) u[k] = 0.0;
-    for (int c = lane; c < dd.chunks; c += 32) {
-        const double* q = pp + (int64_t)c * MAX_RED;
-#pragma unroll
-        for (int k = 0; k < MAX_RED; ++k)
-            if (k < nk) u[k] += q[k];
-    }
-#pragma unroll
-    for (int k = 0; k < MAX_RED; ++k)
-        if (k < nk) {
-            const double t = warp_sum(u[k], dd.chunks);
-            if (lane == 0) cum_out[k] = t;  // scratch until the caller forms the table
+    // p_r = sum over chunks and j < inner of entry r*inner + j (part_src).
+    // Each lane adds its chunks' entries in registers (all loads of a chunk
+    // issued together) and the lanes' sums are combined by the fixed shuffle
+    // tree.
+    const PartSrc ps = part_src(d, dd, b, slot);
+    const int nk = ps.nk, inner = ps.inner;
+    if (pre) {
+        for (int k = lane; k < nk; k += 32) {
+            double t = 0.0;
+            for (int w = 0; w < npre; ++w) t += pre[w][k];
+            cum_out[k] = t;  // scratch until the caller forms the table
         }
+    } else {
+        part_sums(ps, dd.chunks, 0, 1, cum_out);
+    }
     __syncwarp();
     // GB300's float64 pipe retires two lanes per clock per SM, shared by every
     // warp there: each term below is computed by its own lane (the same
@@ -695,10 +728,11 @@ __device__ __forceinline__ bool chained_j2(const DecideDesc& dd) {
 // thresholds; for a chained DEC_KRAUS_J2, the conditional tables
 // p(j | i) = p_ij / sum_j p_ij of every head outcome i (the arithmetic of a
 // separate DEC_KRAUS_J2 decide, row by row)
-__device__ void branch_tables(const DevBatch& d, const DecideDesc& dd, int b, int slot, DecTab& T) {
+__device__ void branch_tables(const DevBatch& d, const DecideDesc& dd, int b, int slot, DecTab& T,
+                              const double (*pre)[MAX_RED] = nullptr, int npre = 0) {
     const int lane = threadIdx.x & 31;
     const bool j2 = chained_j2(dd);
-    warp_probs(d, dd, b, slot, T.p, T.cum, j2 ? T.jp : nullptr);
+    warp_probs(d, dd, b, slot, T.p, T.cum, j2 ? T.jp : nullptr, pre, npre);
     if (lane == 0 && dd.kind != DEC_PAULI) {
         double acc = 0.0;
         for (int r = 0; r < dd.R; ++r) T.cum[r] = (acc += T.p[r]);
@@ -958,6 +992,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 1) k_decide_big(DevBatch d, const
     __shared__ DecTab T;
     __shared__ int ng_sh, nlist_sh;
     __shared__ int list_sh[DEC_THREADS];
+    __shared__ double pre_sh[DEC_THREADS / 32][MAX_RED];
     extern __shared__ __align__(16) unsigned char dec_smem[];
     uint32_t* sm_shot = reinterpret_cast<uint32_t*>(dec_smem);
     uint8_t* sm_key = reinterpret_cast<uint8_t*>(sm_shot + DEC_SPT * DEC_THREADS);
@@ -973,7 +1008,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 1) k_decide_big(DevBatch d, const
         __syncthreads();
         {
             const int64_t bt = b0 + (int64_t)tid * gridDim.x;
-            if (bt < n_br && d.br_count[bt] > DEC_SMALL) list_sh[atomicAdd(&nlist_sh, 1)] = (int)bt;
+            if (bt < n_br && decide_in_cta(dd, d.br_count[bt])) list_sh[atomicAdd(&nlist_sh, 1)] = (int)bt;
         }
         __syncthreads();
         const int nlist = nlist_sh;
@@ -991,7 +1026,12 @@ __global__ void __launch_bounds__(DEC_THREADS, 1) k_decide_big(DevBatch d, const
                 }
             }
             __syncthreads();
-            if (warp == 0) branch_tables(d, dd, b, slot, T);
+            const bool wide = dd.kind != DEC_PAULI && dd.chunks > DEC_WARP_CHUNKS;
+            if (wide) {
+                part_sums(part_src(d, dd, b, slot), dd.chunks, warp, DEC_THREADS / 32, pre_sh[warp]);
+                __syncthreads();
+            }
+            if (warp == 0) branch_tables(d, dd, b, slot, T, wide ? pre_sh : nullptr, DEC_THREADS / 32);
             if (tid < NK) {
                 T.bincnt[tid] = 0;
                 T.binrun[tid] = 0;
@@ -1088,7 +1128,7 @@ __global__ void __launch_bounds__(DECS_WARPS * 32) k_decide_small(DevBatch d, co
     const int gw = blockIdx.x * DECS_WARPS + warp, nw = gridDim.x * DECS_WARPS;
     for (int b = gw; b < n_br; b += nw) {
         const int cnt = *reinterpret_cast<const volatile int32_t*>(&d.br_count[b]);
-        if (cnt > DEC_SMALL) continue;
+        if (decide_in_cta(dd, cnt)) continue;
         // a count the big kernel has just lowered comes after its mark
         __threadfence();
         if (*reinterpret_cast<const volatile int32_t*>(&d.br_big[b]) == (int32_t)dd.op) continue;

@@ -326,6 +326,31 @@ __device__ __forceinline__ void reg_forms1_dyn(const typename Cplx<R>::T* v, int
     }
 }
 
+// A unit's total over the lanes (every lane, fixed tree).  complex64 pairs
+// meet in float-float: GB300's float64 pipe retires two lanes per clock per
+// SM, and a tree of float64 adds for each bin of a 2048-amplitude unit would
+// take half as long as streaming the unit.
+__device__ __forceinline__ double unit_total(Acc<float> a) {
+    float hi = a.hi, lo = a.lo;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float s = __fadd_rn(hi, bh);
+        const float bp = __fsub_rn(s, hi);
+        float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(bh, bp));
+        e = __fadd_rn(e, __fadd_rn(lo, bl));
+        hi = __fadd_rn(s, e);
+        lo = __fsub_rn(e, __fsub_rn(hi, s));
+    }
+    return (double)hi + (double)lo;
+}
+__device__ __forceinline__ double unit_total(Acc<double> a) {
+    double x = a.s;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
 constexpr int REG_MAX_RED = 4;
 constexpr int REG_MAX_BINS = 16;  // measurement outcomes a register pass reduces (k <= 4)
 
@@ -494,22 +519,32 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
     int stride[WP];
 #pragma unroll
     for (int j = 0; j < WP; ++j) stride[j] = 1 << p.tile_q[j];
-    const int64_t units = (int64_t)n_br * p.chunks;
+    // units are 2^k per branch; a warp takes a contiguous range of them.
+    // Without a reduction the units of a branch that fall to the warp are one
+    // run of groups; with one, each unit writes its own partial.
+    const int cshift = __ffs(p.chunks) - 1;
+    const int64_t units = (int64_t)n_br << cshift;
     const int64_t gw = (int64_t)blockIdx.x * nwarps + warp, tw = (int64_t)gridDim.x * nwarps;
     const int64_t u0 = units * gw / tw, u1 = units * (gw + 1) / tw;
-    const int64_t gpu = (d.dim >> WP) / p.chunks;  // groups per unit
+    const int64_t unit_groups = (d.dim >> WP) >> cshift;
     const bool red = p.red_kind != RED_NONE;
     T* const states = reinterpret_cast<T*>(d.states);
     const R* pool = reinterpret_cast<const R*>(d.pool);
-    int cur_b = -1;
-    for (int64_t u = u0; u < u1; ++u) {
-        const int b = (int)(u / p.chunks);
-        const int c = (int)(u % p.chunks);
-        const int slot = d.br_slot[b];
-        if (slot < 0 || slot >= d.n_slots) {
-            if (lane == 0) set_err(d, ERR_SLOT, b);
-            continue;
+    int cur_b = -1, slot = -1;
+    for (int64_t u = u0, ue; u < u1; u = ue) {
+        const int b = (int)(u >> cshift);
+        const int64_t b_end = (int64_t)(b + 1) << cshift;
+        const int64_t c = u - ((int64_t)b << cshift);
+        ue = red ? u + 1 : (b_end < u1 ? b_end : u1);
+        const int64_t gpu = (ue - u) * unit_groups, g0 = c * unit_groups;
+        if (b != cur_b) {
+            slot = d.br_slot[b];
+            if (slot < 0 || slot >= d.n_slots) {
+                if (lane == 0) set_err(d, ERR_SLOT, b);
+                slot = -1;
+            }
         }
+        if (slot < 0) continue;
         if (b != cur_b) {
             const uint64_t clb = d.br_clbits[b];
             // the shared gates' matrices (and the reduction's coefficients)
@@ -674,7 +709,7 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
                 }
                 return bb;
             };
-            const uint32_t base = group_base(c * gpu + gi);
+            const uint32_t base = group_base(g0 + gi);
             T* g = gstate + base;
             auto off = [&](int e) {
                 int o = 0;
@@ -686,7 +721,7 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
             // the lane's next group goes to L2 ahead of its loads (no
             // registers held): the pass is latency-bound at 20 warps per SM
             if (gi + 32 * REG_PREFETCH < gpu) {
-                const T* gn = gstate + group_base(c * gpu + gi + 32 * REG_PREFETCH);
+                const T* gn = gstate + group_base(g0 + gi + 32 * REG_PREFETCH);
 #pragma unroll
                 for (int e = 0; e < G; e += (sizeof(T) == 8 && PAIRED) ? 2 : 1)
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(gn + off(e)));
@@ -758,17 +793,11 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
             }
         }
         if (red && p.red_kind == RED_DIAG) {
-            // the unit's bins (fixed shuffle tree, float64), then every form
-            // from them: lane f writes form f
+            // the unit's bins, then every form from them: lane f writes form f
             const int D = 1 << p.red_k;
             double bin[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                double x = r < D ? acc[r].get() : 0.0;
-                if (r < D)
-                    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                bin[r] = x;
-            }
+            for (int r = 0; r < 4; ++r) bin[r] = r < D ? unit_total(acc[r]) : 0.0;
             if (lane < p.red_R) {
                 const T* W = mats + p.mat_elems - 2 * (p.red_R << p.red_k);
                 double part = 0.0;
@@ -778,23 +807,22 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
                 d.partials[((int64_t)slot * d.max_chunks + c) * MAX_RED + lane] = part;
             }
         } else if (BINS) {
-            // every outcome's bin: a fixed float64 shuffle tree over the lanes
-            for (int r = 0; r < (1 << p.red_k); ++r) {
-                const AS a = bins[r * 32 + lane];
-                double x;
-                if constexpr (sizeof(R) == 4) x = (double)a.x + (double)a.y;
-                else x = a;
-                for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+            for (int r = 0; r < (1 << p.red_k); ++r) {  // every outcome's bin
+                Acc<R> a;
+                if constexpr (sizeof(R) == 4) {
+                    a.hi = bins[r * 32 + lane].x;
+                    a.lo = bins[r * 32 + lane].y;
+                } else {
+                    a.s = bins[r * 32 + lane];
+                }
+                const double x = unit_total(a);
                 if (lane == 0) d.partials[((int64_t)slot * d.max_chunks + c) * MAX_RED + r] = x;
             }
         } else if (red) {
 #pragma unroll
             for (int r = 0; r < REG_MAX_RED; ++r) {
                 if (r >= p.red_R) break;
-                // a unit is short: a float64 shuffle tree costs less here
-                // than float-float pairs
-                double x = acc[r].get();
-                for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+                const double x = unit_total(acc[r]);
                 if (lane == 0) d.partials[((int64_t)slot * d.max_chunks + c) * MAX_RED + r] = x;
             }
         }

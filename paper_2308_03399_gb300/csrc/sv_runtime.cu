@@ -601,10 +601,13 @@ sv_status emit_stages(sv_batch b, const std::vector<int>& idx, const RedSpec& re
         if (std::find(tq.begin(), tq.end(), q) == tq.end()) p.nontile_q[p.n_nontile++] = q;
     p.reg_wp = wp;
     if (wp > 0) {
-        // register path: a warp's unit holds at least REG_UNIT_MIN_AMPS
-        // amplitudes, so the fixed-order combination of its reduction is
-        // paid once per several hundred groups
-        const int64_t unit = std::max<int64_t>(b->dim / b->chunks, REG_UNIT_MIN_AMPS);
+        // register path: with a reduction, a warp's unit holds at least
+        // REG_UNIT_MIN_AMPS amplitudes, so the combination of its sums is
+        // paid once per several groups of every lane; without one, a unit is
+        // one group per lane (a warp runs its units of a branch as one
+        // stretch), so that a few branches still spread over the chip
+        const int64_t unit = red.kind == RED_NONE ? 32ll << wp
+                                                  : std::max<int64_t>(b->dim / b->chunks, REG_UNIT_MIN_AMPS);
         p.chunks = (int)std::max<int64_t>(1, b->dim / unit);
         p.tiles_per_chunk = 1;
     } else {
@@ -2281,7 +2284,7 @@ sv_status sv_alloc_batch(int n_qubits, uint64_t n_shots, int n_clbits, sv_prec p
     b->max_active = DEFAULT_MAX_ACTIVE;
     const int64_t tiles = 1ll << (n_qubits - b->tb);
     b->chunks = (int)std::min<int64_t>(tiles, MAX_CHUNKS);
-    b->chunks_final = (int)std::min<int64_t>(std::max<int64_t>(b->dim / 2048, 1), MAX_CHUNKS);
+    b->chunks_final = (int)std::min<int64_t>(std::max<int64_t>(b->dim / 2048, 1), MAX_FINAL_CHUNKS);
     if (cuda_stream) {
         b->stream = (cudaStream_t)cuda_stream;
     } else {
@@ -2301,8 +2304,6 @@ sv_status sv_alloc_batch(int n_qubits, uint64_t n_shots, int n_clbits, sv_prec p
     // slots
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
-    const int max_chunks = std::max(b->chunks, b->chunks_final);
-    const size_t per_slot = b->state_bytes + (size_t)max_chunks * MAX_RED * 8;
     const size_t per_shot = 4 * 8 + MAX_PEND * 12 + 64;
     const size_t fixed = per_shot * n_shots + (64ull << 20);
     size_t budget = mem_budget;
@@ -2310,9 +2311,16 @@ sv_status sv_alloc_batch(int n_qubits, uint64_t n_shots, int n_clbits, sv_prec p
         const size_t reserve = std::max<size_t>(1ull << 30, total_b / 50);
         budget = free_b > fixed + reserve ? free_b - fixed - reserve : 0;
     }
-    uint64_t slots = budget / per_slot;
-    if (mode == SV_PLAIN) slots = std::min<uint64_t>(slots, 1);
-    else slots = std::min<uint64_t>(slots, n_shots);
+    // the finer chunks only where their partials cost no slot
+    const uint64_t most = mode == SV_PLAIN ? 1 : n_shots;
+    auto slots_with = [&](int chunks) {
+        const size_t per_slot = b->state_bytes + (size_t)std::max(chunks, b->chunks_final) * MAX_RED * 8;
+        return std::min<uint64_t>(budget / per_slot, most);
+    };
+    const int coarse = std::min(b->chunks, MAX_FINAL_CHUNKS);
+    if (slots_with(b->chunks) < slots_with(coarse)) b->chunks = coarse;
+    const int max_chunks = std::max(b->chunks, b->chunks_final);
+    uint64_t slots = slots_with(b->chunks);
     if (slots == 0) {
         sv_free_batch(b);
         return fail(SV_ENOMEM, "not even one state fits the memory budget");
