@@ -59,7 +59,9 @@ cudaError_t launch_resident(const DevBatch& d, int prec, const ResDesc& p, int n
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int grid = n_states < per_sm * n_sm ? n_states : per_sm * n_sm;
-    void* args[] = {(void*)&d, (void*)&p};
+    ResDesc r = p;
+    r.n_states = n_states;
+    void* args[] = {(void*)&d, (void*)&r};
     return cudaLaunchKernel(f, dim3(grid), dim3(threads), args, smem, s);
 }
 

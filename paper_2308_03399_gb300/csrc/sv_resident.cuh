@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resi
     uint8_t* const rows = reinterpret_cast<uint8_t*>(sel_col + MAX_PEND);
     const int2* const index = reinterpret_cast<const int2*>(d.ipool + p.index_off);
     const int2* const batches = reinterpret_cast<const int2*>(d.ipool + p.batch_off);  // first block, blocks
-    const int n_states = d.ctl[CTL_NBR];
+    const int n_states = p.n_states;
 
     // warp w: start the copy of block bt.x + w of a batch
     auto copy_blocks = [&](int2 bt) {
@@ -533,9 +533,28 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resi
         const uint64_t gs = d.shot_base + shot;
         copy_blocks(first);
         if (tid == 0) {
+            const int ps = d.pset_of_shot ? (int)d.pset_of_shot[state] : 0;
             clb_sh = 0;
-            pset_sh = d.br_pset[state];
-            hist_sh = p.hist ? hist_word(0xffffffffu, d.br_pset[state]) : 0ull;
+            pset_sh = ps;
+            hist_sh = p.hist ? hist_word(0xffffffffu, ps) : 0ull;
+            // the branch tables of a run with a state per shot, as a reset
+            // and the run's decides would leave them
+            d.perm[state] = shot;
+            d.br_slot[state] = state;
+            d.br_start[state] = state;
+            d.br_count[state] = 1;
+            d.br_parent[state] = -1;
+            d.br_big[state] = -1;
+            d.br_pset[state] = ps;
+            if (state == 0) {
+                d.ctl[CTL_NBR] = n_states;
+                d.ctl[CTL_NFREE] = 0;  // as many slots as shots
+                d.ctl[CTL_NWAIT] = 0;
+                d.ctl[CTL_COPY_FIRST] = 0;
+                d.ctl[CTL_COPY_END] = 0;
+                d.ctl[CTL_NALLOC] = 0;
+                d.ctl[CTL_DONE] = 0;
+            }
         }
         for (int j = tid; j < dimp; j += nth) {
             T z;
@@ -817,7 +836,10 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resi
                 if (lane == 0) d.keys[shot] = (uint64_t)key;
             }
         }
-        if (tid == 0 && p.hist) p.hist[shot] = hist_sh;
+        if (tid == 0) {
+            d.br_clbits[state] = clb_sh;
+            if (p.hist) p.hist[shot] = hist_sh;
+        }
         __syncthreads();  // st, rows and the block ring are free again
     }
 }

@@ -51,6 +51,7 @@ constexpr int RES_MONO_REAL = 1 << 16;  // a monomial matrix's phases are real (
 
 struct ResDesc {
     int32_t np;           // address bits of the state in shared memory (at least 4)
+    int32_t n_states;     // set at launch
     int32_t n_batches;
     int32_t index_off;    // integer-pool offset of (offset, words) per block
     int32_t batch_off;    // integer-pool offset of (first block, blocks) per batch

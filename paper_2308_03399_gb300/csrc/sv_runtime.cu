@@ -23,6 +23,7 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/sv.h"
@@ -147,6 +148,11 @@ struct sv_batch_s {
     size_t pool_up = 0, ipool_up = 0;
     void* h_pool = nullptr;
     int32_t* h_ipool = nullptr;
+    // one pinned and one device block hold everything of a batch but its
+    // states; the pools move out of them when they grow
+    char* h_block = nullptr;
+    int32_t* h_ctl = nullptr;
+    bool pools_grown = false;
     // scheduler
     std::vector<PendStage> pend;
     uint64_t active = 0;
@@ -296,7 +302,7 @@ int pass_grid(sv_batch b, const PassDesc& p) {
 cudaError_t exec_one(sv_batch b, const Launch& L) {
     const int prec = b->prec == SV_C128;
     switch (L.type) {
-    case L_INIT: return L.a0 == 0 ? cudaSuccess : launch_init(b->dev, prec, L.a0, b->n_sm * 4, b->stream);
+    case L_INIT: return launch_init(b->dev, prec, L.a0, b->n_sm * 4, b->stream);
     case L_RESET: return launch_reset(b->dev, L.a0, L.a1, L.a2, b->n_sm * 2, b->stream);
     case L_PASS:
         if (L.pass.whole) return launch_pass_whole(b->dev, L.pass, pass_grid(b, L.pass), b->stream);
@@ -312,7 +318,6 @@ cudaError_t exec_one(sv_batch b, const Launch& L) {
 }
 
 int launch_kernels(const Launch& L) {
-    if (L.type == L_INIT && L.a0 == 0) return 0;
     return L.type == L_FINAL ? 3 : (L.type == L_DECIDE ? 2 : 1);
 }
 
@@ -354,6 +359,14 @@ sv_status emit(sv_batch b, Launch&& L) {
 }
 
 // ---- pool ------------------------------------------------------------------
+void free_pools(sv_batch b) {
+    if (!b->pools_grown) return;  // parts of the batch's blocks
+    cudaFree(b->d_pool);
+    cudaFreeHost(b->h_pool);
+    cudaFree(b->d_ipool);
+    cudaFreeHost(b->h_ipool);
+}
+
 // grow the device pool and its pinned staging copy (everything is uploaded
 // again afterwards)
 sv_status grow_pool(sv_batch b) {
@@ -370,10 +383,8 @@ sv_status grow_pool(sv_batch b) {
         cudaFree(di);
         return fail(SV_ENOMEM, "cannot grow the constant pool");
     }
-    cudaFree(b->d_pool);
-    cudaFreeHost(b->h_pool);
-    cudaFree(b->d_ipool);
-    cudaFreeHost(b->h_ipool);
+    free_pools(b);
+    b->pools_grown = true;
     b->d_pool = dp;
     b->h_pool = hp;
     b->d_ipool = (int32_t*)di;
@@ -1410,10 +1421,17 @@ sv_status op_final(sv_batch b, uint32_t op) {
     return emit(b, std::move(L));
 }
 
+// the control words, through pinned memory (waits for the stream)
+sv_status read_ctl(sv_batch b, int32_t* ctl) {
+    CU(cudaMemcpyAsync(b->h_ctl, b->dev.ctl, sizeof(int32_t) * CTL_WORDS, cudaMemcpyDeviceToHost, b->stream));
+    CU(cudaStreamSynchronize(b->stream));
+    memcpy(ctl, b->h_ctl, sizeof(int32_t) * CTL_WORDS);
+    return SV_OK;
+}
+
 sv_status check_device_error(sv_batch b) {
     int32_t ctl[CTL_WORDS];
-    CU(cudaMemcpyAsync(ctl, b->dev.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, b->stream));
-    CU(cudaStreamSynchronize(b->stream));
+    if (sv_status st = read_ctl(b, ctl)) return st;
     if (ctl[CTL_ERR] == ERR_TIMEOUT) return fail(SV_ETIMEOUT, "device wait timed out");
     if (ctl[CTL_ERR] != 0) {
         char buf[128];
@@ -1423,11 +1441,6 @@ sv_status check_device_error(sv_batch b) {
     return SV_OK;
 }
 
-sv_status read_ctl(sv_batch b, int32_t* ctl) {
-    CU(cudaMemcpyAsync(ctl, b->dev.ctl, sizeof(int32_t) * CTL_WORDS, cudaMemcpyDeviceToHost, b->stream));
-    CU(cudaStreamSynchronize(b->stream));
-    return SV_OK;
-}
 
 // the end of a round of a logged shot-branching run: keep the shot
 // permutation (a fork event's shot set is a range of it, valid until the
@@ -1469,8 +1482,21 @@ sv_status circuit_op(sv_batch b, const sv_circuit* c, int i) {
     return fail(SV_EINVAL, "unknown op kind");
 }
 
+// four independent lanes of 8 bytes: a byte-wise hash's multiply chain took
+// longer than a small circuit's kernels (70 us for the 54 KB of tables of a
+// 10-qubit, depth-20 brickwork)
 uint64_t fnv(uint64_t h, const void* p, size_t n) {
     const unsigned char* c = (const unsigned char*)p;
+    uint64_t a[4] = {h, h + 0x9E3779B97F4A7C15ull, h + 0xC2B2AE3D27D4EB4Full, h + 0x165667B19E3779F9ull};
+    for (; n >= 32; n -= 32, c += 32)
+        for (int j = 0; j < 4; ++j) {
+            uint64_t w;
+            memcpy(&w, c + 8 * j, 8);
+            a[j] = (a[j] ^ w) * 0x9FB21C651E98DF25ull;
+            a[j] ^= a[j] >> 32;
+        }
+    h = a[0];
+    for (int j = 1; j < 4; ++j) h = (h ^ a[j]) * 1099511628211ull + (h >> 29);
     for (size_t i = 0; i < n; ++i) h = (h ^ c[i]) * 1099511628211ull;
     return h;
 }
@@ -1486,6 +1512,9 @@ uint64_t circuit_hash(sv_batch b, const sv_circuit* c) {
     h = fnv(h, c->d_off, 8 * n);
     h = fnv(h, c->cond_clbit, 4 * n);
     h = fnv(h, c->cond_val, 4 * n);
+    h = fnv(h, c->reset, 4 * n);
+    for (size_t i = 0; i < n; ++i)
+        if (c->kind[i] == SV_OP_MEASURE) h = fnv(h, c->clbits + c->cl_off[i], 4 * (size_t)c->nq[i]);
     int64_t dmax = 0, qmax = 0;
     for (size_t i = 0; i < n; ++i) qmax = std::max<int64_t>(qmax, c->q_off[i] + c->nq[i]);
     h = fnv(h, c->qubits, 4 * qmax);
@@ -2347,30 +2376,63 @@ sv_status sv_alloc_batch(int n_qubits, uint64_t n_shots, int n_clbits, sv_prec p
     b->allocs.push_back(states);
     d.states = states;
     const uint64_t S = n_shots;
-    if ((st = dalloc(b, &d.ctl, CTL_WORDS)) || (st = dalloc(b, &d.br_slot, S)) || (st = dalloc(b, &d.br_start, S)) ||
-        (st = dalloc(b, &d.br_count, S)) || (st = dalloc(b, &d.br_clbits, S)) || (st = dalloc(b, &d.br_parent, S)) || (st = dalloc(b, &d.br_big, S)) || (st = dalloc(b, &d.br_pset, S)) ||
-        (st = dalloc(b, &d.br_sel, S * MAX_PEND)) || (st = dalloc(b, &d.br_scale, S * MAX_PEND)) ||
-        (st = dalloc(b, &d.perm, S)) || (st = dalloc(b, &d.perm_tmp, S)) || (st = dalloc(b, &d.shot_sel, S)) ||
-        (st = dalloc(b, &d.free_slots, b->n_slots)) || (st = dalloc(b, &d.wait_shots, S)) ||
-
-        (st = dalloc(b, &d.partials, (size_t)b->n_slots * max_chunks * MAX_RED)) || (st = dalloc(b, &d.keys, S)) ||
-        (st = dalloc(b, &d.pass_log, 1 << 20)) || (st = dalloc(b, &d.pos_branch, S))) {
-        sv_free_batch(b);
-        return st;
-    }
     b->pool_cap = 1 << 16;
     b->ipool_cap = 1 << 14;
-    if (cudaMalloc(&b->d_pool, b->pool_cap * 8) != cudaSuccess ||
-        cudaMalloc((void**)&b->d_ipool, b->ipool_cap * 4) != cudaSuccess ||
-        cudaMallocHost(&b->h_pool, b->pool_cap * 8) != cudaSuccess ||
-        cudaMallocHost((void**)&b->h_ipool, b->ipool_cap * 4) != cudaSuccess) {
+    d.pass_log_cap = 1 << 20;
+    // one allocation: measured on GB300, some 20 separate ones and their
+    // frees took most of a small per-op run's time
+    char* base = nullptr;
+    size_t size = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        size_t off = 0;
+        auto part = [&](auto** q, size_t count) {
+            if (base) *q = reinterpret_cast<std::remove_reference_t<decltype(*q)>>(base + off);
+            off += (std::max<size_t>(count, 1) * sizeof(**q) + 255) & ~(size_t)255;
+        };
+        part(&d.ctl, CTL_WORDS);
+        part(&d.br_slot, S);
+        part(&d.br_start, S);
+        part(&d.br_count, S);
+        part(&d.br_clbits, S);
+        part(&d.br_parent, S);
+        part(&d.br_big, S);
+        part(&d.br_pset, S);
+        part(&d.br_sel, S * MAX_PEND);
+        part(&d.br_scale, S * MAX_PEND);
+        part(&d.perm, S);
+        part(&d.perm_tmp, S);
+        part(&d.shot_sel, S);
+        part(&d.free_slots, b->n_slots);
+        part(&d.wait_shots, S);
+        part(&d.partials, (size_t)b->n_slots * max_chunks * MAX_RED);
+        part(&d.keys, S);
+        part(&d.pass_log, d.pass_log_cap);
+        part(&d.pos_branch, S);
+        double* pool = nullptr;
+        part(&pool, b->pool_cap);
+        part(&b->d_ipool, b->ipool_cap);
+        b->d_pool = pool;
+        if (pass == 0) {
+            size = off;
+            if (cudaMalloc((void**)&base, size) != cudaSuccess) {
+                cudaGetLastError();
+                sv_free_batch(b);
+                return fail(SV_ENOMEM, "cannot allocate the batch's tables");
+            }
+            b->allocs.push_back(base);
+        }
+    }
+    const size_t hp = b->pool_cap * 8, hi = b->ipool_cap * 4;
+    if (cudaMallocHost((void**)&b->h_block, hp + hi + 256) != cudaSuccess) {
         cudaGetLastError();
         sv_free_batch(b);
         return fail(SV_ENOMEM, "cannot allocate the constant pool");
     }
+    b->h_pool = b->h_block;
+    b->h_ipool = (int32_t*)(b->h_block + hp);
+    b->h_ctl = (int32_t*)(b->h_block + hp + hi);
     d.pool = b->d_pool;
     d.ipool = b->d_ipool;
-    d.pass_log_cap = 1 << 20;
     if (init_kernels() != cudaSuccess || init_resident() != cudaSuccess) {
         sv_free_batch(b);
         return fail(SV_ECUDA, "cannot configure the kernels");
@@ -2392,10 +2454,8 @@ sv_status sv_free_batch(sv_batch b) {
         cudaEventDestroy(e.second.second);
     }
     for (void* p : b->allocs) cudaFree(p);
-    if (b->d_pool) cudaFree(b->d_pool);
-    if (b->d_ipool) cudaFree(b->d_ipool);
-    if (b->h_pool) cudaFreeHost(b->h_pool);
-    if (b->h_ipool) cudaFreeHost(b->h_ipool);
+    free_pools(b);
+    if (b->h_block) cudaFreeHost(b->h_block);
     if (b->side) {
         cudaStreamSynchronize(b->side);
         cudaStreamDestroy(b->side);
@@ -2564,8 +2624,7 @@ sv_status sv_branch(sv_batch b, uint32_t op) {
 sv_status sv_get_keys(sv_batch b, uint64_t* keys) {
     if (!b || !keys) return fail(SV_EINVAL, "NULL argument");
     CU(cudaMemcpyAsync(keys, b->dev.keys, b->n_shots * 8, cudaMemcpyDeviceToHost, b->stream));
-    CU(cudaStreamSynchronize(b->stream));
-    return check_device_error(b);
+    return check_device_error(b);  // waits for the stream
 }
 
 static sv_status histogram(sv_batch b, uint64_t* keys, uint64_t* counts, uint64_t cap, uint64_t* n_out) {
@@ -2658,16 +2717,18 @@ sv_status sv_run_circuit(sv_batch b, const sv_circuit* c, int use_graph) {
     int n_run = (int)b->n_shots;
     if ((st = tree_begin(b))) return st;
     for (int round = 0;; ++round) {
-        Launch r;
-        r.type = L_RESET;
-        r.a0 = branch;
-        r.a1 = n_run;
-        r.a2 = from_wait;
-        if ((st = exec(b, r))) return st;
-        Launch in;
-        in.type = L_INIT;
-        in.a0 = resident ? 0 : root_slots(b, n_run);
-        if ((st = exec(b, in))) return st;
+        if (!resident) {  // a resident launch resets the batch by itself
+            Launch r;
+            r.type = L_RESET;
+            r.a0 = branch;
+            r.a1 = n_run;
+            r.a2 = from_wait;
+            if ((st = exec(b, r))) return st;
+            Launch in;
+            in.type = L_INIT;
+            in.a0 = root_slots(b, n_run);
+            if ((st = exec(b, in))) return st;
+        }
         if (use_graph && !resident) {
             if (!cached && round == 0) {
                 if (b->graph_exec) {
@@ -2799,15 +2860,19 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
             std::vector<Launch>& L = b0->multi_lists[i];
             std::vector<Launch> ops;
             if ((st = record_circuit(bs[i], cs[i], ops))) return st;
+            if (is_resident(ops)) {
+                L = ops;
+                continue;
+            }
             Launch r;
             r.type = L_RESET;
-            r.a0 = bs[i]->branch && !is_resident(ops);
+            r.a0 = bs[i]->branch;
             r.a1 = (int)bs[i]->n_shots;
             r.a2 = 0;
             L.push_back(r);
             Launch in;
             in.type = L_INIT;
-            in.a0 = is_resident(ops) ? 0 : root_slots(bs[i], (int)bs[i]->n_shots);
+            in.a0 = root_slots(bs[i], (int)bs[i]->n_shots);
             L.push_back(in);
             L.insert(L.end(), ops.begin(), ops.end());
         }
