@@ -109,6 +109,54 @@ __device__ __noinline__ void stage_dense(typename Cplx<R>::T* tile, int tb, cons
     }
 }
 
+// A matrix that is mostly zeros (the density-matrix method's channels: 28 of
+// the 256 entries of a two-qubit depolarizing superoperator): rows[r] has bit
+// c set where entry (r, c) is nonzero, and the products of the others, exact
+// zeros, are left out.  complex128 runs on a float64 pipe of two lanes per
+// clock per SM, where the dense product of one 16 x 16 stage on an 18-qubit
+// state takes 30 us of the whole chip.  A group's rows are shared by `split`
+// threads of one warp, which read before any of them writes.
+template <class R, int K>
+__device__ __noinline__ void stage_sparse(typename Cplx<R>::T* tile, int tb, const int32_t* pos,
+                                          const typename Cplx<R>::T* M, const uint32_t* rows) {
+    using T = typename Cplx<R>::T;
+    constexpr int D = 1 << K, SPLIT = K >= 4 ? 4 : 2, RN = D / SPLIT;
+    const GroupIdx<K> gi(pos);
+    const int items = SPLIT << (tb - K);
+    for (int i0 = 0; i0 < items; i0 += blockDim.x) {
+        const int i = i0 + threadIdx.x;
+        const bool on = i < items;
+        const int base = insert_zeros<K>(on ? i / SPLIT : 0, gi.sp), r0 = (i % SPLIT) * RN;
+        T out[RN];
+        if (on) {
+            T v[D];
+#pragma unroll
+            for (int r = 0; r < D; ++r) v[r] = tile[base | gi.off[r]];
+#pragma unroll
+            for (int q = 0; q < RN; ++q) {
+                T acc;
+                acc.x = 0;
+                acc.y = 0;
+                const uint32_t m = rows[r0 + q];
+#pragma unroll
+                for (int c = 0; c < D; ++c)
+                    if ((m >> c) & 1) cfma(acc, M[(r0 + q) * D + c], v[c]);
+                out[q] = acc;
+            }
+        }
+        __syncwarp();
+        if (on)
+#pragma unroll
+            for (int q = 0; q < RN; ++q) {
+                int o = 0;
+#pragma unroll
+                for (int j = 0; j < K; ++j)
+                    if (((r0 + q) >> j) & 1) o |= 1 << pos[j];
+                tile[base | o] = out[q];
+            }
+    }
+}
+
 // Pauli string from its parameters (Section IV-A-3): bit flips x, phase
 // flips z, number of Y; out[d] = (-i)^ny (-1)^popcount(z & d) in[d ^ x].
 template <class R, int K>
@@ -173,8 +221,11 @@ __device__ __noinline__ void stage_proj(typename Cplx<R>::T* tile, int tb, const
 template <class R>
 __device__ __forceinline__ void stage_dispatch(typename Cplx<R>::T* tile, int tb, const Stage& st,
                                                const typename Cplx<R>::T* M, int sel, double scale, int packed,
-                                               int mono) {
-    if (mono) {
+                                               int mono, const uint32_t* rows) {
+    if (rows) {
+        if (st.k == 3) stage_sparse<R, 3>(tile, tb, st.pos, M, rows);
+        else stage_sparse<R, 4>(tile, tb, st.pos, M, rows);
+    } else if (mono) {
         stage_mono<R>(tile, tb, st.pos, mono, M);
     } else if (st.kind == ST_DENSE || st.kind == ST_DENSE_BR) {
         if (st.k == 1) stage_dense<R, 1>(tile, tb, st.pos, M);
@@ -359,6 +410,7 @@ __global__ void __launch_bounds__(256, 2) k_pass(DevBatch d, const __grid_consta
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw + ((pass_bytes_before_bars(p, blockDim.x, sizeof(T)) + 7) & ~7ull));
     __shared__ int skip[MAX_STAGES], sel_sh[MAX_STAGES], packed_sh[MAX_STAGES], mono_sh[MAX_STAGES];
     __shared__ double scale_sh[MAX_STAGES];
+    __shared__ uint32_t rows_sh[MAX_STAGES][16];  // nonzero columns per row of 3- and 4-qubit matrices
     __shared__ double wsum[8][MAX_RED];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -505,9 +557,25 @@ __global__ void __launch_bounds__(256, 2) k_pass(DevBatch d, const __grid_consta
                 mono_sh[st_i] = mi;
             }
             if (first)
-                for (int st_i = threadIdx.x; st_i < p.n_stages; st_i += blockDim.x)
-                    if (p.st[st_i].k != 2 || (p.st[st_i].kind != ST_DENSE && p.st[st_i].kind != ST_DENSE_BR))
-                        mono_sh[st_i] = 0;
+                for (int st_i = threadIdx.x; st_i < p.n_stages; st_i += blockDim.x) {
+                    const Stage& st = p.st[st_i];
+                    if (st.k == 2 && (st.kind == ST_DENSE || st.kind == ST_DENSE_BR)) continue;
+                    mono_sh[st_i] = 0;
+                    if (st.kind != ST_DENSE || (st.k != 3 && st.k != 4)) continue;
+                    // at most a quarter of the entries nonzero: by rows
+                    const int D = 1 << st.k;
+                    int nz = 0;
+                    for (int r = 0; r < D; ++r) {
+                        uint32_t m = 0;
+                        for (int c = 0; c < D; ++c) {
+                            const T x = mats[st.mat + r * D + c];
+                            if (x.x != 0 || x.y != 0) m |= 1u << c;
+                        }
+                        rows_sh[st_i][r] = m;
+                        nz += __popc(m);
+                    }
+                    if (4 * nz <= D * D) mono_sh[st_i] = -1;
+                }
             __syncthreads();
             cur_b = b;
         }
@@ -523,7 +591,9 @@ __global__ void __launch_bounds__(256, 2) k_pass(DevBatch d, const __grid_consta
         for (int st_i = 0; st_i < p.n_stages; ++st_i) {
             if (skip[st_i]) continue;
             const Stage& st = p.st[st_i];
-            stage_dispatch<R>(tile, tb, st, mats + st.mat, sel_sh[st_i], scale_sh[st_i], packed_sh[st_i], mono_sh[st_i]);
+            const int mono = mono_sh[st_i];
+            stage_dispatch<R>(tile, tb, st, mats + st.mat, sel_sh[st_i], scale_sh[st_i], packed_sh[st_i],
+                              mono < 0 ? 0 : mono, mono < 0 ? rows_sh[st_i] : nullptr);
             __syncthreads();
         }
         if (red) reduce_dispatch<R>(tile, tb, p, mats + p.mat_elems - 2 * (p.red_R << (2 * p.red_k)), acc);
