@@ -115,6 +115,7 @@ struct DecideDesc {
     int32_t clbit[MAX_STAGE_Q];
     int32_t r2;                // joint Kraus: terms of the second op (partials stride)
     int32_t pend_prev;         // DEC_KRAUS_J2: pending column of the first op's choice
+    int32_t c64;               // complex64 states
     uint64_t live_cols;        // choice columns whose stages are still pending (forks copy them)
     int32_t* log_sel;          // per shot id, nullable
     double* log_thr;           // 2 per shot id, nullable

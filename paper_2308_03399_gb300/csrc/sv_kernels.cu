@@ -661,17 +661,6 @@ __global__ void __launch_bounds__(256, 2) k_pass(DevBatch d, const __grid_consta
 constexpr int DEC_THREADS = 512;
 constexpr int DEC_SMALL = 64;
 
-// Sum over the lanes by a fixed xor tree.  Lanes at or past `used` hold
-// exact zeros, and adding a zero changes nothing, so the tree can start at
-// the level that first mixes the used lanes: the same result in fewer
-// float64 adds (each a 16-cycle FP64-pipe instruction on GB300).
-__device__ __forceinline__ double warp_sum(double x, int used) {
-    int o = 16;
-    while (o > 1 && o >= used) o >>= 1;
-    for (; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
 // per-branch tables of one decide (shared memory: one per warp or per CTA)
 struct DecTab {
     double p[MAX_TERMS], cum[MAX_TERMS];  // head op: probabilities, running sums
@@ -707,25 +696,26 @@ __device__ __forceinline__ PartSrc part_src(const DevBatch& d, const DecideDesc&
     return {d.partials + (int64_t)src * d.max_chunks * MAX_RED + base_r, dd.R * inner, inner};
 }
 
-// this warp's share (chunks w, w + nw, ... in blocks of 32) of the sums of a
-// branch's terms, into out[0..nk) (lane 0)
+// this warp's share of the sums of a branch's terms, into out[0..nk).  Lanes
+// are (chunk, term): a lane adds its term over every 32 / K-th chunk (K: nk
+// rounded up to a power of two) and the lanes of a term meet in log2(32 / K)
+// float64 adds for all terms at once.  The decides of some thousand branches
+// are bound by the float64 pipe (two lanes per clock per SM, 16 clocks an
+// instruction), where a tree per term took several times as many.
 __device__ __forceinline__ void part_sums(const PartSrc& ps, int chunks, int w, int nw, double* out) {
     const int lane = threadIdx.x & 31;
-    double u[MAX_RED];
-#pragma unroll
-    for (int k = 0; k < MAX_RED; ++k) u[k] = 0.0;
-    for (int c = 32 * w + lane; c < chunks; c += 32 * nw) {
-        const double* q = ps.pp + (int64_t)c * MAX_RED;
-#pragma unroll
-        for (int k = 0; k < MAX_RED; ++k)
-            if (k < ps.nk) u[k] += q[k];
+    const int kb = ps.nk <= 1 ? 0 : 32 - __clz(ps.nk - 1), K = 1 << kb, per = 32 >> kb;
+    const int k = lane & (K - 1), c0 = w * per + (lane >> kb);
+    double u = 0.0;
+    if (k < ps.nk) {
+        const double* q = ps.pp + k;
+#pragma unroll 4
+        for (int c = c0; c < chunks; c += per * nw) u += q[(int64_t)c * MAX_RED];
     }
-#pragma unroll
-    for (int k = 0; k < MAX_RED; ++k)
-        if (k < ps.nk) {
-            const double t = warp_sum(u[k], chunks - 32 * w < 0 ? 0 : chunks - 32 * w);
-            if (lane == 0) out[k] = t;
-        }
+    // lanes of chunks past the last hold exact zeros: only the levels that
+    // mix used lanes
+    for (int o = K; o < 32 && (o >> kb) < chunks - w * per; o <<= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+    if (lane < ps.nk) out[lane] = u;
 }
 
 // Branches whose sums run over more chunks than this take a CTA whatever
@@ -790,6 +780,13 @@ __device__ void warp_probs(const DevBatch& d, const DecideDesc& dd, int b, int s
     __syncwarp();
 }
 
+// 1 / sqrt(p).  complex64 rounds it to float32 before use: the float64
+// reciprocal square root (within an ulp) gives the same factor at a third of
+// the float64 instructions of a root and a division.
+__device__ __forceinline__ double scale_of(const DecideDesc& dd, double p) {
+    return dd.c64 ? rsqrt(p) : 1.0 / sqrt(p);
+}
+
 __device__ __forceinline__ bool chained_j2(const DecideDesc& dd) {
     return dd.n_tail > 0 && dd.tail[0].kind == DEC_KRAUS_J2;
 }
@@ -826,13 +823,13 @@ __device__ void branch_tables(const DevBatch& d, const DecideDesc& dd, int b, in
             double acc = 0.0;
             for (int jj = 0; jj <= j; ++jj) acc += T.jp[i * R2 + jj];
             T.jcum[lane] = acc;
-            T.jsc[lane] = 1.0 / sqrt(T.jp[lane]);
+            T.jsc[lane] = scale_of(dd, T.jp[lane]);
         }
     }
     __syncwarp();
     for (int r = lane; r < dd.R; r += 32) {
         T.thr[r] = cum_threshold(T.cum[r]);
-        T.sc[r] = dd.kind == DEC_PAULI ? 1.0 : 1.0 / sqrt(T.p[r]);
+        T.sc[r] = dd.kind == DEC_PAULI ? 1.0 : scale_of(dd, T.p[r]);
     }
     if (j2)
         for (int k = lane; k < dd.R * dd.tail[0].R; k += 32) T.jthr[k] = cum_threshold(T.jcum[k]);

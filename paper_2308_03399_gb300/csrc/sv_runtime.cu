@@ -1013,6 +1013,7 @@ sv_status emit_decide(sv_batch b, uint32_t op, int kind, int R, const double* cu
     d.pend_prev = pend_prev;
     d.nk = R;
     d.live_cols = b->col_used;
+    d.c64 = b->prec == SV_C64;
     for (int j = 0; j < m; ++j) d.clbit[j] = clbits[j];
     if (cum)
         for (int t = 0; t < R; ++t) d.cum[t] = cum[t];
