@@ -116,6 +116,7 @@ struct DecideDesc {
     int32_t r2;                // joint Kraus: terms of the second op (partials stride)
     int32_t pend_prev;         // DEC_KRAUS_J2: pending column of the first op's choice
     int32_t c64;               // complex64 states
+    int32_t max_cnt;           // no branch has more shots than this
     uint64_t live_cols;        // choice columns whose stages are still pending (forks copy them)
     int32_t* log_sel;          // per shot id, nullable
     double* log_thr;           // 2 per shot id, nullable
@@ -128,6 +129,19 @@ struct DecideDesc {
     double tail_cum[MAX_TAIL_TERMS];
     uint64_t tail_thr[MAX_TAIL_TERMS];  // ceil(cum * 2^53), see cum_threshold
 };
+
+// Branches of more than DEC_SMALL shots, and those whose sums run over more
+// chunks than DEC_WARP_CHUNKS, are decided by a CTA (a warp adding the 8192
+// chunks of a 27-qubit state needs longer than a small state's whole pass),
+// the others by a warp.
+constexpr int DEC_SMALL = 64;
+constexpr int DEC_WARP_CHUNKS = 512;
+
+// the decide kernels that can have work: 1 per warp, 2 per CTA, 3 both
+inline int decide_kernels(const DecideDesc& dd) {
+    if (dd.kind != DEC_PAULI && dd.chunks > DEC_WARP_CHUNKS) return 2;
+    return dd.max_cnt <= DEC_SMALL ? 1 : 3;
+}
 
 struct FinalDesc {
     uint32_t op;
@@ -195,12 +209,11 @@ enum : int32_t {
 
 // launchers (sv_kernels.cu)
 cudaError_t launch_init(const DevBatch& d, int prec, int n_init_slots, int grid, cudaStream_t s);
-cudaError_t launch_reset(const DevBatch& d, int mode_branch, int n_shots_run, int from_wait, int grid,
-                         cudaStream_t s);
+cudaError_t launch_reset(const DevBatch& d, int mode_branch, int n_shots_run, int from_wait, int n_rows, int table,
+                         int grid, cudaStream_t s);
 cudaError_t launch_pass(const DevBatch& d, int prec, const PassDesc& p, int threads, int grid, cudaStream_t s);
 cudaError_t launch_decide(const DevBatch& d, const DecideDesc& dd, int n_sm, cudaStream_t s, cudaStream_t side,
                           cudaEvent_t ev_fork, cudaEvent_t ev_join);
-cudaError_t launch_predraw(const DevBatch& d, int n_rows, int table, int n_shots, int grid, cudaStream_t s);
 cudaError_t launch_copy(const DevBatch& d, int prec, int grid, cudaStream_t s);
 cudaError_t launch_final(const DevBatch& d, int prec, const FinalDesc& f, int grid, cudaStream_t s);
 size_t pass_smem_bytes(int prec, const PassDesc& p, int threads);

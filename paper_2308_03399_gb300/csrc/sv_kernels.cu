@@ -23,7 +23,7 @@
 //                   group a branch id and a free slot (or park its shots on
 //                   the waiting list when none is left).  The small- and
 //                   big-branch kernels run side by side.
-//   k_predraw       batch mode: every shot's Pauli choices, before the gates.
+//   k_reset         run start; batch mode: every shot's Pauli choices too.
 //   k_copy          copy parent states into the new branches' slots.
 //   k_final_*       sampling of all qubits from each branch (sampling measure).
 //
@@ -659,7 +659,6 @@ __global__ void __launch_bounds__(256, 2) k_pass(DevBatch d, const __grid_consta
 // (k_decide_small).
 // ---------------------------------------------------------------------------
 constexpr int DEC_THREADS = 512;
-constexpr int DEC_SMALL = 64;
 
 // per-branch tables of one decide (shared memory: one per warp or per CTA)
 struct DecTab {
@@ -718,10 +717,6 @@ __device__ __forceinline__ void part_sums(const PartSrc& ps, int chunks, int w, 
     if (lane < ps.nk) out[lane] = u;
 }
 
-// Branches whose sums run over more chunks than this take a CTA whatever
-// their shots: a warp adding the 8192 chunks of a 27-qubit state needs
-// longer than a small state's whole pass
-constexpr int DEC_WARP_CHUNKS = 512;
 __device__ __forceinline__ bool decide_in_cta(const DecideDesc& dd, int cnt) {
     return cnt > DEC_SMALL || (dd.kind != DEC_PAULI && dd.chunks > DEC_WARP_CHUNKS);
 }
@@ -1246,8 +1241,8 @@ __global__ void __launch_bounds__(DECS_WARPS * 32) k_decide_small(DevBatch d, co
 }
 
 // ---------------------------------------------------------------------------
-// k_predraw: Pauli choices of every shot for the Pauli ops of a batch-mode
-// circuit, drawn before the first gate (Section IV-A-3 samples Pauli noise
+// predraw_rows: Pauli choices of every shot for the Pauli ops of a batch-mode
+// circuit, drawn by the reset before the first gate (Section IV-A-3 samples Pauli noise
 // ahead of applying it).  With one shot per branch a Pauli choice never
 // forks anything, so no decide is needed: row q of pre_sel holds op q's
 // choice per shot id, and the pass reads its branch's shot's entry.  The
@@ -1259,7 +1254,7 @@ __device__ __forceinline__ uint64_t ipool_u64(const int32_t* ip, int64_t off) {
     return (uint64_t)(uint32_t)ip[off] | ((uint64_t)(uint32_t)ip[off + 1] << 32);
 }
 
-__global__ void __launch_bounds__(256) k_predraw(DevBatch d, int n_rows, int table, int n_shots) {
+__device__ __forceinline__ void predraw_rows(const DevBatch& d, int n_rows, int table, int n_shots) {
     const int64_t total = (int64_t)n_rows * n_shots;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
@@ -1276,11 +1271,6 @@ __global__ void __launch_bounds__(256) k_predraw(DevBatch d, int n_rows, int tab
         double* log_thr = reinterpret_cast<double*>(ipool_u64(d.ipool, table + (int64_t)PRE_WORDS * q + 6));
         log_choice(log_sel, log_thr, s, sel, cum);
     }
-}
-
-cudaError_t launch_predraw(const DevBatch& d, int n_rows, int table, int n_shots, int grid, cudaStream_t s) {
-    k_predraw<<<grid, 256, 0, s>>>(d, n_rows, table, n_shots);
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -1425,7 +1415,8 @@ __global__ void k_wait_snapshot(DevBatch d) { d.ctl[CTL_NRUN] = d.ctl[CTL_NWAIT]
 
 // from_wait: 0 shots 0 .. n_run-1; 1 the first n_run waiting shots; 2 every
 // waiting shot (count from the device)
-__global__ void __launch_bounds__(256) k_reset(DevBatch d, int branch_mode, int n_run, int from_wait) {
+__global__ void __launch_bounds__(256) k_reset(DevBatch d, int branch_mode, int n_run, int from_wait, int n_rows,
+                                               int table) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (from_wait == 2) n_run = d.ctl[CTL_NRUN];
@@ -1457,6 +1448,7 @@ __global__ void __launch_bounds__(256) k_reset(DevBatch d, int branch_mode, int 
         d.ctl[CTL_NALLOC] = 0;
         d.ctl[CTL_DONE] = 0;
     }
+    if (n_rows > 0) predraw_rows(d, n_rows, table, n_run);
 }
 
 // Shot-branching with a parameter sweep: shots with different parameters
@@ -1612,9 +1604,20 @@ cudaError_t launch_decide(const DevBatch& d, const DecideDesc& dd, int n_sm, cud
     // count drops to DEC_SMALL or fewer is marked before its count changes,
     // so the small kernel never decides it again (br_big).  Both kernels are
     // latency-bound and grid-stride over the branches, so each launches
-    // exactly one resident wave.
+    // exactly one resident wave.  Where every branch falls to one of them,
+    // only that one is launched, on the batch's stream: without the fork and
+    // join a decide is one node instead of a diamond.
     static const int small_per_sm = resident_blocks((const void*)k_decide_small, DECS_WARPS * 32);
     static const int big_per_sm = resident_blocks((const void*)k_decide_big, DEC_THREADS, DEC_BIG_SMEM);
+    const int which = decide_kernels(dd);
+    if (which == 1) {
+        k_decide_small<<<small_per_sm * n_sm, DECS_WARPS * 32, 0, s>>>(d, dd);
+        return cudaGetLastError();
+    }
+    if (which == 2) {
+        k_decide_big<<<big_per_sm * n_sm, DEC_THREADS, DEC_BIG_SMEM, s>>>(d, dd);
+        return cudaGetLastError();
+    }
     cudaError_t e = cudaEventRecord(ev_fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ev_fork, 0);
     if (e != cudaSuccess) return e;
@@ -1625,8 +1628,6 @@ cudaError_t launch_decide(const DevBatch& d, const DecideDesc& dd, int n_sm, cud
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev_join, 0);
     return e;
 }
-
-
 
 cudaError_t launch_copy(const DevBatch& d, int prec, int grid, cudaStream_t s) {
     const int64_t vec16 = d.dim * (prec ? 16 : 8) / 16;
@@ -1653,11 +1654,11 @@ cudaError_t launch_init(const DevBatch& d, int prec, int n_init_slots, int grid,
     return cudaGetLastError();
 }
 
-cudaError_t launch_reset(const DevBatch& d, int mode_branch, int n_shots_run, int from_wait, int grid,
-                         cudaStream_t s) {
+cudaError_t launch_reset(const DevBatch& d, int mode_branch, int n_shots_run, int from_wait, int n_rows, int table,
+                         int grid, cudaStream_t s) {
     if (from_wait == 2) k_wait_snapshot<<<1, 1, 0, s>>>(d);
     if (mode_branch && d.pset_of_shot) k_reset_psets<<<1, RESET_PSET_THREADS, 0, s>>>(d, n_shots_run, from_wait);
-    else k_reset<<<grid, 256, 0, s>>>(d, mode_branch, n_shots_run, from_wait);
+    else k_reset<<<grid, 256, 0, s>>>(d, mode_branch, n_shots_run, from_wait, n_rows, table);
     return cudaGetLastError();
 }
 

@@ -8,7 +8,7 @@
 // state (Kraus, measurement), when the pass would exceed its fusion width,
 // or when the state is read.  Pauli choices do not depend on the state
 // (Section IV-A-3) and are sampled without touching it: in batch mode all
-// of them up front (k_predraw), otherwise by a decide.  A decide that
+// of them up front (by the reset), otherwise by a decide.  A decide that
 // follows another with no pass between joins it as a chain, and in
 // shot-branching mode each decide is followed by k_copy, so no host
 // synchronisation happens inside a circuit (Section IV-A-4).
@@ -64,12 +64,13 @@ struct PreRow {
     double* log_thr;
 };
 
-enum LType { L_INIT, L_RESET, L_PASS, L_DECIDE, L_ALLOC, L_COPY, L_FINAL, L_PREDRAW, L_RESIDENT };
+enum LType { L_INIT, L_RESET, L_PASS, L_DECIDE, L_ALLOC, L_COPY, L_FINAL, L_RESIDENT };
 enum PClass { P_PASS = 0, P_DECIDE, P_ALLOC, P_COPY, P_FINAL, P_INIT, P_OTHER, P_N };
 
 struct Launch {
     LType type;
     int a0 = 0, a1 = 0, a2 = 0;
+    int pre_rows = 0, pre_table = 0;  // L_RESET: Pauli ops drawn up front
     uint32_t op = 0;
     PassDesc pass;
     DecideDesc dec;
@@ -204,6 +205,7 @@ struct sv_batch_s {
     bool predraw = true;  // batch mode: Pauli choices drawn up front, no decides
     std::vector<PreRow> pre_rows;  // of the circuit being recorded
     int pre_cap = 0;               // rows the device table holds
+    int predraw_rows = 0, predraw_table = 0;  // of the recorded circuit: drawn by its reset
     std::map<int, int> reg_occ;
     int slot_limit = 0;
     // resident runs (k_resident): options that shape the pass kernels and
@@ -253,7 +255,6 @@ int pclass(LType t) {
     case L_PASS: return P_PASS;
     case L_RESIDENT: return P_PASS;
     case L_DECIDE: return P_DECIDE;
-    case L_PREDRAW: return P_DECIDE;
     case L_ALLOC: return P_ALLOC;
     case L_COPY: return P_COPY;
     case L_FINAL: return P_FINAL;
@@ -303,7 +304,8 @@ cudaError_t exec_one(sv_batch b, const Launch& L) {
     const int prec = b->prec == SV_C128;
     switch (L.type) {
     case L_INIT: return launch_init(b->dev, prec, L.a0, b->n_sm * 4, b->stream);
-    case L_RESET: return launch_reset(b->dev, L.a0, L.a1, L.a2, b->n_sm * 2, b->stream);
+    case L_RESET:
+        return launch_reset(b->dev, L.a0, L.a1, L.a2, L.pre_rows, L.pre_table, b->n_sm * (L.pre_rows ? 4 : 2), b->stream);
     case L_PASS:
         if (L.pass.whole) return launch_pass_whole(b->dev, L.pass, pass_grid(b, L.pass), b->stream);
         return launch_pass(b->dev, prec, L.pass, tile_threads(b, L.pass), pass_grid(b, L.pass), b->stream);
@@ -311,14 +313,13 @@ cudaError_t exec_one(sv_batch b, const Launch& L) {
     case L_ALLOC: return cudaSuccess;
     case L_COPY: return launch_copy(b->dev, prec, b->n_sm * 4, b->stream);
     case L_FINAL: return launch_final(b->dev, prec, L.fin, b->grid_small, b->stream);
-    case L_PREDRAW: return launch_predraw(b->dev, L.a0, L.a1, L.a2, b->n_sm * 4, b->stream);
     case L_RESIDENT: return launch_resident(b->dev, prec, L.res, L.a1, b->n_sm, b->stream);
     }
     return cudaErrorInvalidValue;
 }
 
 int launch_kernels(const Launch& L) {
-    return L.type == L_FINAL ? 3 : (L.type == L_DECIDE ? 2 : 1);
+    return L.type == L_FINAL ? 3 : (L.type == L_DECIDE && decide_kernels(L.dec) == 3 ? 2 : 1);
 }
 
 void count_launch(sv_batch b, const Launch& L) {
@@ -1014,6 +1015,7 @@ sv_status emit_decide(sv_batch b, uint32_t op, int kind, int R, const double* cu
     d.nk = R;
     d.live_cols = b->col_used;
     d.c64 = b->prec == SV_C64;
+    d.max_cnt = b->branch ? (int)std::min<uint64_t>(b->n_shots, 1ull << 30) : 1;
     for (int j = 0; j < m; ++j) d.clbit[j] = clbits[j];
     if (cum)
         for (int t = 0; t < R; ++t) d.cum[t] = cum[t];
@@ -1023,11 +1025,11 @@ sv_status emit_decide(sv_batch b, uint32_t op, int kind, int R, const double* cu
         // per-op call in shot-branching mode (Section IV-B-2's sample, then
         // branch): this launch draws and logs every shot's choice; the same
         // keyed draws fork the branches when sv_branch commits
+        // (without a log nobody sees the choices before that: nothing to launch)
         b->commit = L;
         d.sample_only = 1;
         d.fork = 0;
-        st = emit(b, std::move(L));
-        if (st) return st;
+        if (b->log && (st = emit(b, std::move(L)))) return st;
         b->uncommitted = true;
         b->last_random = op;
         return SV_OK;
@@ -1166,7 +1168,7 @@ sv_status op_pauli(sv_batch b, uint32_t op, int k, const int* q, int n_terms, co
     }
     if ((st = ensure_started(b))) return st;
     // batch mode, whole circuits: the choice of every shot is drawn up front
-    // (k_predraw), so the op needs no decide and no pending column
+    // (by the reset), so the op needs no decide and no pending column
     const bool pre = b->rec && !b->branch && b->predraw &&
                      (b->rec_resident || (uint64_t)(b->pre_rows.size() + 1) * b->n_shots <= PRE_TABLE_BYTES);
     if ((st = make_room(b, q, k, 0, !pre))) return st;
@@ -1672,8 +1674,8 @@ sv_status run_plain(sv_batch b, const sv_circuit* c) {
 // the launch sequence of a whole circuit (without the reset / init of the
 // root), with its constants uploaded
 // the pre-drawn rows of a recorded circuit: their descriptors go to the
-// integer pool, the device table grows to hold them, and the draw is the
-// circuit's first launch
+// integer pool, the device table grows to hold them, and the run's reset
+// draws them
 int push_row_table(sv_batch b) {
     const int table = (int)b->ipool.size();
     for (const PreRow& r : b->pre_rows) {
@@ -1685,7 +1687,7 @@ int push_row_table(sv_batch b) {
     return table;
 }
 
-sv_status finish_predraw(sv_batch b, std::vector<Launch>& launches) {
+sv_status finish_predraw(sv_batch b) {
     const int n = (int)b->pre_rows.size();
     const int table = push_row_table(b);
     if (n > b->pre_cap) {
@@ -1694,12 +1696,8 @@ sv_status finish_predraw(sv_batch b, std::vector<Launch>& launches) {
         b->pre_cap = n;
         b->pool_gen += 1;  // kernels take the batch by value
     }
-    Launch L;
-    L.type = L_PREDRAW;
-    L.a0 = n;
-    L.a1 = table;
-    L.a2 = (int)b->n_shots;
-    launches.insert(launches.begin(), L);
+    b->predraw_rows = n;
+    b->predraw_table = table;
     return SV_OK;
 }
 
@@ -2225,6 +2223,7 @@ sv_status record_ops(sv_batch b, const sv_circuit* c, std::vector<Launch>& launc
 
 sv_status record_circuit(sv_batch b, const sv_circuit* c, std::vector<Launch>& launches) {
     const bool candidate = resident_candidate(b), branch = b->branch;
+    b->predraw_rows = 0;
     b->rec_resident = candidate;
     if (candidate) b->branch = false;  // every shot its own branch
     sv_status st = record_ops(b, c, launches);
@@ -2238,7 +2237,7 @@ sv_status record_circuit(sv_batch b, const sv_circuit* c, std::vector<Launch>& l
             (st = record_ops(b, c, launches)))
             return st;
     }
-    if (!b->pre_rows.empty() && (st = finish_predraw(b, launches))) return st;
+    if (!b->pre_rows.empty() && (st = finish_predraw(b))) return st;
     return upload_pool(b);
 }
 
@@ -2724,6 +2723,8 @@ sv_status sv_run_circuit(sv_batch b, const sv_circuit* c, int use_graph) {
             r.a0 = branch;
             r.a1 = n_run;
             r.a2 = from_wait;
+            r.pre_rows = b->predraw_rows;
+            r.pre_table = b->predraw_table;
             if ((st = exec(b, r))) return st;
             Launch in;
             in.type = L_INIT;
@@ -2870,6 +2871,8 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
             r.a0 = bs[i]->branch;
             r.a1 = (int)bs[i]->n_shots;
             r.a2 = 0;
+            r.pre_rows = bs[i]->predraw_rows;
+            r.pre_table = bs[i]->predraw_table;
             L.push_back(r);
             Launch in;
             in.type = L_INIT;
