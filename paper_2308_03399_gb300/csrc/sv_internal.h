@@ -218,6 +218,7 @@ cudaError_t launch_copy(const DevBatch& d, int prec, int grid, cudaStream_t s);
 cudaError_t launch_final(const DevBatch& d, int prec, const FinalDesc& f, int grid, cudaStream_t s);
 size_t pass_smem_bytes(int prec, const PassDesc& p, int threads);
 size_t pass_reg_smem_bytes(int prec, const PassDesc& p, int threads);
+bool pass_fold_fits(const PassDesc& p);
 int pass_reg_blocks_per_sm(int prec, int wp, int paired, int var, size_t smem);
 int pass_reg_variant(int prec, const PassDesc& p);
 // register pass kernel instantiations (one translation unit per group)

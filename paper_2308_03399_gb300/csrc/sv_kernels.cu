@@ -1535,6 +1535,12 @@ cudaError_t init_kernels() {
         e = cudaFuncSetAttribute(k_pass<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_decide_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DEC_BIG_SMEM);
+    // a folded pass at the limit of pass_fold_fits, with its work area
+    for (int wp = 1; wp <= 4; ++wp)
+        for (int paired = 0; paired < 2; ++paired)
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(reg_kernel_fold_c64(wp, paired), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         64 * 1024);
     return e;
 }
 
@@ -1564,12 +1570,18 @@ int pass_reg_blocks_per_sm(int prec, int wp, int paired, int var, size_t smem) {
     return n > 0 ? n : 1;
 }
 
+// Whether a pass may fold does not depend on how the composition is laid out:
+// the matrices, a G x G slice per warp and the stage words within 48 KB
+bool pass_fold_fits(const PassDesc& p) {
+    const size_t nw = RegCta<float>::threads / 32, m = (size_t)((p.mat_elems + 1) & ~1), g = (size_t)1 << p.reg_wp;
+    return nw * (m * 24 + 4 * MAX_STAGES * 4 + g * g * 8) <= 48 * 1024;
+}
+
 size_t pass_reg_smem_bytes(int prec, const PassDesc& p, int threads) {
     const size_t c = prec ? 16 : 8;
     const size_t nw = threads / 32;
     const size_t m = (size_t)((p.mat_elems + 1) & ~1);
-    const size_t g = (size_t)1 << p.reg_wp;
-    return nw * (m * c + 4 * MAX_STAGES * 4) + (prec ? 0 : nw * m * 16) + (p.fold && !prec ? nw * g * g * 8 : 0) +
+    return nw * (m * c + 4 * MAX_STAGES * 4) + (prec ? 0 : nw * m * 16) + (p.fold && !prec ? nw * (8 * FOLD_LD * 16 + MAX_STAGES * 16) : 0) +
            (p.red_kind == RED_BINS ? nw * REG_MAX_BINS * 32 * 8 : 0);
 }
 

@@ -5,6 +5,7 @@
 #pragma once
 
 #include "sv_common.cuh"
+#include "sv_fold.cuh"
 
 namespace sv {
 
@@ -426,7 +427,7 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     // shared memory, each region one slice per warp: matrices | stage
     // choice, packed form, scale (4 x MAX_STAGES words) | complex64 only:
-    // the matrices expanded for packed FMAs | the folded matrix (G x G)
+    // the matrices expanded for packed FMAs | the folded matrix, its stages
     const int mat_stride = (p.mat_elems + 1) & ~1;
     T* const mats_all = reinterpret_cast<T*>(smem_raw);
     int* const words_all = reinterpret_cast<int*>(mats_all + (size_t)nwarps * mat_stride);
@@ -436,7 +437,11 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
     int* w_packed = w_sel + MAX_STAGES;
     double* w_scale = reinterpret_cast<double*>(w_sel + 2 * MAX_STAGES);
     ulonglong2* matx = matx_all + (size_t)warp * mat_stride;
-    float4* fold_m = reinterpret_cast<float4*>(matx_all + (size_t)nwarps * mat_stride) + (size_t)warp * (G / 2) * G;
+    // folded passes: the work matrix (the folded matrix, see res_compose)
+    // and the list of active stages
+    float4* const fold_all = reinterpret_cast<float4*>(matx_all + (size_t)nwarps * mat_stride);
+    float4* fold_m = fold_all + (size_t)warp * 8 * FOLD_LD;
+    int4* fold_act = reinterpret_cast<int4*>(fold_all + (size_t)nwarps * 8 * FOLD_LD) + (size_t)warp * MAX_STAGES;
     // measurement bins (RED_BINS): per warp, bin r of lane l at bins[r * 32 + l]
     // (float-float pairs for complex64), after the folded matrices (none in
     // a pass with a reduction) and, for complex64, the expanded matrices
@@ -672,22 +677,34 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
             }
             __syncwarp();
             if constexpr (FOLD && sizeof(T) == 8) {
-                // lane c < G runs the stages on the unit vector e_c: its
-                // result is column c of the pass's matrix for this branch
-                T col[G];
-#pragma unroll
-                for (int e = 0; e < G; ++e) {
-                    col[e].x = e == lane ? (R)1 : (R)0;
-                    col[e].y = 0;
+                // the active stages as a list, then composed on the unit
+                // vectors (a lane running every register layout of a stage
+                // took some 2000 clocks a stage, most of it instruction
+                // fetch)
+                int count = 0;
+                for (int s0 = 0; s0 < p.n_stages; s0 += 32) {
+                    const int s = s0 + lane;
+                    const bool on = s < p.n_stages && !((skipmask >> s) & 1);
+                    const unsigned m = __ballot_sync(0xffffffffu, on);
+                    if (on) {
+                        const Stage& st = p.st[s];
+                        int4 a = make_int4(RA_PROJ, 0, w_packed[s], 0);
+                        const unsigned char* mat = reinterpret_cast<const unsigned char*>(mats + st.mat);
+                        if (st.kind == ST_DENSE || st.kind == ST_DENSE_BR) {
+                            if (st.k == 1) a.x = a.z ? RA_ONE_SHAPED : RA_ONE;
+                            else a.x = a.z ? RA_MONO : RA_TWO;
+                            if (a.x == RA_TWO) mat = reinterpret_cast<const unsigned char*>(matx + st.mat);
+                        } else if (st.kind == ST_PAULI_BR) {
+                            a.x = RA_PAULI;
+                        }
+                        a.y = (int)(mat - smem_raw);
+                        for (int j = 0; j < st.k; ++j) a.w |= st.pos[j] << (4 * j);
+                        fold_act[count + __popc(m & ((1u << lane) - 1u))] = a;
+                    }
+                    count += __popc(m);
                 }
-                apply_stages(col);
-                // rows r and r + 1 of column c side by side: one 128-bit
-                // load per column serves two output rows
-                if (lane < G)
-#pragma unroll
-                    for (int r = 0; r < G; r += 2)
-                        fold_m[(r / 2) * G + lane] = make_float4(col[r].x, col[r].y, col[r + 1].x, col[r + 1].y);
                 __syncwarp();
+                res_compose(fold_act, count, smem_raw, reinterpret_cast<float2*>(fold_m));
             }
             cur_b = b;
         }
@@ -742,7 +759,7 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
             }
             if constexpr (FOLD && sizeof(T) == 8) {
                 // the pass's stages folded into one G x G matrix (rows r and
-                // r + 1 of column c at fold_m[(r / 2) * G + c]); a folded pass
+                // r + 1 of column c at fold_m[(r / 2) * FOLD_LD + c]); a folded pass
                 // has no reduction, so each pair of output rows is stored as
                 // soon as it is formed
 #pragma unroll 1
@@ -750,7 +767,7 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
                     float2 o0 = make_float2(0.f, 0.f), o1 = make_float2(0.f, 0.f);
 #pragma unroll
                     for (int c2 = 0; c2 < G; ++c2) {
-                        const float4 m = fold_m[(r / 2) * G + c2];
+                        const float4 m = fold_m[(r / 2) * FOLD_LD + c2];
                         const float2 a = v[c2];
                         o0.x = fmaf(m.x, a.x, fmaf(-m.y, a.y, o0.x));
                         o0.y = fmaf(m.x, a.y, fmaf(m.y, a.x, o0.y));

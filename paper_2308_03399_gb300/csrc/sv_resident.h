@@ -44,9 +44,6 @@ enum : int32_t {
     RD_KIND = 0, RD_R, RD_PEND, RD_OP, RD_R2, RD_OP2, RD_PEND2, RD_M, RD_CLBITS, RD_WORDS
 };
 
-// entries of the active-stage list
-enum : int32_t { RA_ONE = 0, RA_ONE_SHAPED, RA_TWO, RA_MONO, RA_PAULI, RA_PROJ };
-
 constexpr int RES_MONO_REAL = 1 << 16;  // a monomial matrix's phases are real (with its mono_info)
 
 struct ResDesc {

@@ -673,7 +673,7 @@ sv_status emit_stages(sv_batch b, const std::vector<int>& idx, const RedSpec& re
     p.mat_elems = mat;
     if (wp > 0 && b->fold && b->prec == SV_C64 && red.kind == RED_NONE && p.store && fold_pays(b, ss, wp)) {
         p.fold = 1;
-        if (pass_reg_smem_bytes(0, p, pass_reg_threads(0)) > 48 * 1024) p.fold = 0;
+        if (!pass_fold_fits(p)) p.fold = 0;
     }
     // the rest of the queue stays pending
     std::vector<PendStage> rest;
