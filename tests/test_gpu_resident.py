@@ -142,3 +142,33 @@ def test_resident_parameter_sweep(prec):
     assert np.array_equal(k1[:40], [O.run_shot(oc, 9, s, pset=int(ps[s]))["key"] for s in range(40)])
     ref = O.run_shot(oc, 9, 0, want_state=True, pset=int(ps[0]))["state"]
     assert np.abs(a[0] - ref).max() <= AMP[prec]
+
+
+@pytest.mark.parametrize("name,prec", [("n5_kraus", sv.SV_C64), ("n5_kraus", sv.SV_C128), ("n8_mid4", sv.SV_C64),
+                                       ("n9_qft", sv.SV_C64), ("n9_qft", sv.SV_C128), ("n13_brick", sv.SV_C64)])
+def test_resident_branching_runs_match_passes(name, prec):
+    # a shot-branching batch with a slot per shot: the same keys and states,
+    # and sv_stats reports the branches and fork copies the run stands for
+    c = CIRCUITS[name]()
+    n = 300
+    k1, k2, a, st = _run(c, prec, sv.SV_BRANCH, n, 78)
+    p1, _, pa, pst = _run(c, prec, sv.SV_BRANCH, n, 78, [(sv.SV_OPT_MAX_ACTIVE, 4)])
+    assert st["launches"] < 5 < pst["launches"], "the run was not resident"
+    assert np.array_equal(k1, k2) and np.array_equal(k1, p1)
+    assert st["live_branches"] == pst["live_branches"] and st["copy_bytes"] == pst["copy_bytes"]
+    if prec == sv.SV_C64:
+        assert all(np.array_equal(x, y) for x, y in zip(a, pa))
+    else:
+        assert all(np.abs(x - y).max() <= AMP[prec] for x, y in zip(a, pa))
+
+
+def test_short_of_slots_stays_on_passes():
+    # fewer slots than shots: the waiting list, as without resident runs
+    c = CIRCUITS["n7_su4"]()
+    with sv.Batch(c.n_qubits, 200, 1, sv.SV_C64, sv.SV_BRANCH, 79) as b:
+        b.set_option(sv.SV_OPT_SLOT_LIMIT, 20)
+        b.run_circuit(sv.circuit_struct(c.to_arrays()), use_graph=True)
+        st, keys = b.stats(), b.get_keys()
+    assert st["restarts"] > 0
+    oc = O.OracleCircuit(c)
+    assert np.array_equal(keys[:20], [O.run_shot(oc, 79, s)["key"] for s in range(20)])
