@@ -29,6 +29,14 @@
 // then apply the blocks one after another, and warp 0 decides the reduction.
 // The next batch's blocks are on their way to shared memory (cp.async)
 // meanwhile.
+//
+// Measured on GB300, us a run, passes -> resident: 6-qubit brickwork x 100
+// shots 169 -> 74, 10-qubit x 1000 829 -> 292, 13-qubit QFT x 4000 6550 ->
+// 2500, 12-qubit QFT with Kraus noise x 4000 (shot-branching passes) 30700 ->
+// 16700, 11-qubit complex128 sweep x 1000 2680 -> 2250.  What bounds it: issue
+// slots (42% used at 12 qubits, some 7000 warp instructions a Kraus pass) and
+// barriers in complex64, the float64 pipe (two lanes per clock per SM) in
+// complex128.
 #pragma once
 #include <cuda_runtime.h>
 

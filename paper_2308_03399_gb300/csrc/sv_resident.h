@@ -67,6 +67,7 @@ struct ResDesc {
 inline int res_swz(int a) { return a ^ ((a >> 4) & 15) ^ ((a >> 8) & 15) ^ ((a >> 12) & 15); }
 
 int resident_threads(int prec, int np);
+inline bool resident_one_cta(int prec, int np) { return np >= (prec ? 13 : 14); }  // per SM
 int resident_batch(int prec, int np);  // most blocks of a batch
 size_t resident_smem_bytes(int prec, const ResDesc& p);
 cudaError_t init_resident();

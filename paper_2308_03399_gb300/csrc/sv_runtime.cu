@@ -1718,7 +1718,9 @@ bool resident_candidate(sv_batch b) {
 
 // Shot-branching shares the states of shots that agree so far but pays a
 // decide, a copy and a pass launch per random op; a resident run simulates
-// every shot by itself in one launch.  Both are estimated in microseconds
+// every shot by itself in one launch (12-qubit SU(4) x 4000: 2.6 ms branching
+// and 3.8 ms resident at noise 1e-4, 4.2 and 3.8 ms at 3e-2; 12-qubit QFT x
+// 4000: 5.7 and 1.6 ms, 9.0 and 1.7 ms).  Both are estimated in microseconds
 // from GB300 timings (circuits of 6 to 13 qubits, 100 to 4000 shots,
 // noise of 1e-4 to 3e-2): the
 // branching run from its launches and the number of live branches that the
@@ -2116,6 +2118,16 @@ bool build_resident(sv_batch b, std::vector<Launch>& launches) {
     ResDesc r;
     memset(&r, 0, sizeof(r));
     r.np = std::max(4, b->n);
+    // states that leave room for one CTA per SM: its latency is hidden by
+    // nothing else, so over many waves passes with a reduction come out even
+    // and complex128 ones behind (14-qubit SU(4), 100 shots 4.06 ms on passes
+    // and 0.70 resident, 2000 shots 9.5 and 8.9; 13-qubit complex128
+    // mid-circuit measurements, 100 shots 7.4 and 1.9 ms, 2000 21.4 and 25.5)
+    if (resident_one_cta(b->prec == SV_C128, r.np) && b->n_shots > (uint64_t)4 * b->n_sm) {
+        bool red = b->prec == SV_C128;
+        for (const Launch& L : launches) red = red || (L.type == L_PASS && L.pass.red_kind != RED_NONE);
+        if (red) return false;
+    }
     std::vector<std::vector<int32_t>> blocks;
     int n_passes = 0;
     bool ok = (int)b->pre_rows.size() <= RES_MAX_ROWS;
