@@ -623,11 +623,13 @@ sv_status emit_stages(sv_batch b, const std::vector<int>& idx, const RedSpec& re
         p.chunks = (int)std::max<int64_t>(1, b->dim / unit);
         p.tiles_per_chunk = 1;
     } else {
-        // tile path: a chunk spans at least eight tiles (or the whole
-        // state), so the fixed-order combination of its reduction is paid
-        // once per several tiles
+        // tile path: with a reduction, a chunk spans at least eight tiles (or
+        // the whole state), so the fixed-order combination of its sums is
+        // paid once per several tiles; without one every tile is a unit of
+        // its own (eight a unit left an 18-qubit density matrix on 32 CTAs:
+        // 227 us a pass)
         const int64_t tiles = 1ll << (b->n - p.tb);
-        const int64_t tpc = std::max<int64_t>(tiles / b->chunks, std::min<int64_t>(tiles, 8));
+        const int64_t tpc = red.kind == RED_NONE ? 1 : std::max<int64_t>(tiles / b->chunks, std::min<int64_t>(tiles, 8));
         p.chunks = (int)(tiles / tpc);
         p.tiles_per_chunk = (int)tpc;
     }
