@@ -327,26 +327,11 @@ __device__ __forceinline__ void reg_forms1_dyn(const typename Cplx<R>::T* v, int
     }
 }
 
-// A unit's total over the lanes (every lane, fixed tree).  complex64 pairs
-// meet in float-float: GB300's float64 pipe retires two lanes per clock per
-// SM, and a tree of float64 adds for each bin of a 2048-amplitude unit would
-// take half as long as streaming the unit.
-__device__ __forceinline__ double unit_total(Acc<float> a) {
-    float hi = a.hi, lo = a.lo;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
-        const float s = __fadd_rn(hi, bh);
-        const float bp = __fsub_rn(s, hi);
-        float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(bh, bp));
-        e = __fadd_rn(e, __fadd_rn(lo, bl));
-        hi = __fadd_rn(s, e);
-        lo = __fsub_rn(e, __fsub_rn(hi, s));
-    }
-    return (double)hi + (double)lo;
-}
-__device__ __forceinline__ double unit_total(Acc<double> a) {
-    double x = a.s;
+// A unit's total over the lanes (every lane, fixed tree), in float64: with
+// units of 8192 amplitudes a tree of float-float pairs (14 instructions a
+// level) cost 2.5 ms of the 87 ms of passes of a 16-qubit SU(4) run more than this one.
+template <class R> __device__ __forceinline__ double unit_total(const Acc<R>& a) {
+    double x = a.get();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
