@@ -121,8 +121,11 @@ __device__ __forceinline__ void res_diag(const typename Cplx<R>::T* v, int run, 
 }
 
 // one selection by a whole warp: lane r < R holds the probability of outcome
-// r; the running sums, the integer thresholds and the fallback are those of
-// select_k
+// r.  Thresholds and fallback are those of select_k; the running sums come
+// from a scan (four float64 adds where 16 outcomes one after another cost a
+// 367-pass Kraus run 4%), so a sum can differ from select_k's in its last bits
+// and exceed its neighbour's for an outcome of probability 0.  Such an outcome
+// is never drawn: only those with p > 0 are candidates.
 __device__ __forceinline__ int warp_select(double p, int R, uint64_t k53) {
     const int lane = threadIdx.x & 31;
     double c = lane < R ? p : 0.0;
@@ -130,10 +133,10 @@ __device__ __forceinline__ int warp_select(double p, int R, uint64_t k53) {
         const double y = __shfl_up_sync(0xffffffffu, c, o);
         if (lane >= o) c += y;
     }
-    const double prev = __shfl_up_sync(0xffffffffu, c, 1);
-    unsigned m = __ballot_sync(0xffffffffu, lane < R && k53 < cum_threshold(c));
+    const bool possible = lane < R && p > 0.0;
+    unsigned m = __ballot_sync(0xffffffffu, possible && k53 < cum_threshold(c));
     if (m) return __ffs(m) - 1;
-    m = __ballot_sync(0xffffffffu, lane < R && c > (lane ? prev : 0.0));
+    m = __ballot_sync(0xffffffffu, possible);
     return m ? 31 - __clz(m) : R - 1;
 }
 
