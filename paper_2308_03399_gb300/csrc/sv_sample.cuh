@@ -5,12 +5,12 @@
 //
 // A state of 2^n amplitudes is cut into `chunks` contiguous chunks of L
 // amplitudes.  chunk_sum() / chunk_sum_warp() give one chunk's sum of
-// |psi_j|^2 (one CTA or one warp, float-float or float64 per lane, fixed-order
-// combination); chunk_cum()
+// |psi_j|^2 (one CTA or one warp, float-float or float64 per lane, the lanes
+// combined to float64 precision in a fixed order); chunk_cum()
 // turns a state's chunk sums into a running sum (one warp, fixed order);
 // sample_warp() draws one key: the chunk by a two-level warp search over the
 // running sums, then the first j with u < C_j by a warp prefix sum over 256
-// amplitudes at a time (8 per lane), all in float64.
+// amplitudes at a time (8 per lane), to float64 precision.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -50,12 +50,51 @@ template <class R> struct Cx;
 template <> struct Cx<float> { using T = float2; };
 template <> struct Cx<double> { using T = double2; };
 
+// A sum in three float32 words, each TwoSum's error carried on to the next
+// word: value() is it rounded to float64 once, so sums kept this way lose no
+// more than float64 ones.  complex64 sums of a warp meet in this form: the
+// float64 pipe retires two lanes per clock per SM (16 clocks an instruction),
+// a merge is 21 float32 instructions on a pipe of 128.
+struct Sum3 {
+    float hi = 0.f, mid = 0.f, lo = 0.f;
+    static __device__ __forceinline__ float two_sum(float& a, float x) {
+        const float s = __fadd_rn(a, x), bp = __fsub_rn(s, a);
+        const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(x, bp));
+        a = s;
+        return e;
+    }
+    __device__ __forceinline__ void add_mid(float x) { lo = __fadd_rn(lo, two_sum(mid, x)); }
+    __device__ __forceinline__ void add_sq(float x) {
+        const float p = __fmul_rn(x, x);
+        add_mid(two_sum(hi, p));
+        add_mid(__fmaf_rn(x, x, -p));
+    }
+};
+__device__ __forceinline__ void merge(Sum3& a, const Sum3& b) {  // the same bits for (b, a)
+    const float e = Sum3::two_sum(a.hi, b.hi), f = Sum3::two_sum(a.mid, b.mid), g = Sum3::two_sum(a.mid, e);
+    a.lo = __fadd_rn(__fadd_rn(a.lo, b.lo), __fadd_rn(f, g));
+}
+__device__ __forceinline__ void merge(double& a, double b) { a += b; }
+__device__ __forceinline__ Sum3 lane_xor(const Sum3& a, int o) {
+    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.mid, o),
+            __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ double lane_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ double value(const Sum3& a) { return (double)a.hi + ((double)a.mid + (double)a.lo); }
+__device__ __forceinline__ double value(double a) { return a; }
+
+// the warp's sum (every lane; fixed order)
+template <class W> __device__ __forceinline__ double warp_sum(W a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) merge(a, lane_xor(a, o));
+    return value(a);
+}
+
 template <class R> struct Sum;
 template <> struct Sum<double> {
     double s = 0.0;
     __device__ __forceinline__ void add_sq(double x, double y) { s += x * x + y * y; }
-    __device__ __forceinline__ void merge_xor(int o) { s += __shfl_xor_sync(0xffffffffu, s, o); }
-    __device__ __forceinline__ double get() const { return s; }
+    __device__ __forceinline__ double wide() const { return s; }
 };
 // float-float pair (Knuth's TwoSum); the squares of float32 values enter
 // exactly: x*x rounded plus its error fma(x, x, -x*x) (Dekker's product)
@@ -75,27 +114,8 @@ template <> struct Sum<float> {
         add(py);
         lo = __fadd_rn(lo, __fadd_rn(ex, ey));
     }
-    // plus the pair of lane ^ o (TwoSum of the high words, renormalised)
-    __device__ __forceinline__ void merge_xor(int o) {
-        const float bh = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
-        const float s = __fadd_rn(hi, bh);
-        const float bp = __fsub_rn(s, hi);
-        float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(bh, bp));
-        e = __fadd_rn(e, __fadd_rn(lo, bl));
-        hi = __fadd_rn(s, e);
-        lo = __fsub_rn(e, __fsub_rn(hi, s));
-    }
-    __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
+    __device__ __forceinline__ Sum3 wide() const { return {hi, lo, 0.f}; }
 };
-
-// the warp's sum (every lane; fixed order).  float-float pairs meet on the
-// float32 pipe: float64 adds retire two lanes per clock per SM, and a tree of
-// them for every 16 KB of amplitudes costs more than reading them
-template <class R> __device__ __forceinline__ double warp_sum_of(Sum<R> a) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a.merge_xor(o);
-    return a.get();
-}
 
 // amplitudes j and j + 1 (j even): one 128-bit load where the state starts on
 // a 16-byte boundary
@@ -142,7 +162,7 @@ __device__ __forceinline__ void sum_strided(Sum<R>& a, const typename Cx<R>::T* 
 template <class R> __device__ __forceinline__ double chunk_sum_warp(const typename Cx<R>::T* g, int64_t L) {
     Sum<R> a;
     sum_strided<R>(a, g, L, threadIdx.x & 31, 32);
-    return warp_sum_of<R>(a);
+    return warp_sum(a.wide());
 }
 
 // chunks of at most this many amplitudes take a warp each (no block barrier,
@@ -154,7 +174,7 @@ template <class R>
 __device__ __forceinline__ double chunk_sum(const typename Cx<R>::T* g, int64_t L, double* sh32) {
     Sum<R> a;
     sum_strided<R>(a, g, L, threadIdx.x, blockDim.x);
-    const double x = warp_sum_of<R>(a);
+    const double x = warp_sum(a.wide());
     __syncthreads();
     if ((threadIdx.x & 31) == 0) sh32[threadIdx.x >> 5] = x;
     __syncthreads();
@@ -236,12 +256,24 @@ __device__ __forceinline__ int64_t sample_warp(const typename Cx<R>::T* g, int64
         const int64_t j0 = (int64_t)c * L;
         for (int64_t blk = 0; blk < L && key < 0; blk += 256) {
             if constexpr (sizeof(R) == 4) {
-                // the block's total on the float32 pipe; the float64 prefix
-                // below only for the block that holds the draw
+                // the block's total (some 500 float32 instructions, where
+                // float64 takes 45 of 16 clocks); the running sums below
+                // only for the block that holds the draw
                 if (L > 256) {
-                    Sum<R> t;
-                    sum_strided<R>(t, g + j0 + blk, 256, lane, 32);
-                    const double tot = warp_sum_of<R>(t);
+                    const typename Cx<R>::T* gb = g + j0 + blk;
+                    const bool aligned = (reinterpret_cast<uintptr_t>(gb) & 15) == 0;
+                    float4 v[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[k] = load_pair(gb + 2 * (lane + 32 * k), aligned);
+                    Sum3 t;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        t.add_sq(v[k].x);
+                        t.add_sq(v[k].y);
+                        t.add_sq(v[k].z);
+                        t.add_sq(v[k].w);
+                    }
+                    const double tot = warp_sum(t);
                     if (!(u < acc + tot) && blk + 256 < L) {
                         acc += tot;
                         continue;
