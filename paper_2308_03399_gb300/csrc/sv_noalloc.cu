@@ -29,7 +29,6 @@ namespace {
 
 constexpr int NA_MAX_DEVICES = 64;
 constexpr size_t NA_SCRATCH_DOUBLES = 131072;  // 1 MiB
-constexpr int NA_MAX_CHUNKS = 1024;  // chunk count limit (as in the batch path)
 
 static __device__ __align__(256) double na_scratch[NA_SCRATCH_DOUBLES];
 
@@ -47,6 +46,7 @@ __global__ void __launch_bounds__(256) na_partials(const typename svs::Cx<R>::T*
         [&](int64_t it, double s) { scratch[it] = s; });
 }
 
+// per state (one warp): running sum of its chunk sums, in place
 __global__ void __launch_bounds__(256) na_cum(int chunks, int n_states, double* scratch) {
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     for (int st = gw; st < n_states; st += nw)
@@ -86,8 +86,7 @@ extern "C" sv_status sv_final_sample_noalloc(const void* states, sv_prec prec, i
         return SV_EINVAL;
     }
     const int64_t dim = 1ll << n_qubits;
-    const int64_t c0 = dim / 2048;
-    const int chunks = (int)(c0 < 1 ? 1 : (c0 > NA_MAX_CHUNKS ? NA_MAX_CHUNKS : c0));
+    const int chunks = svs::final_chunks(dim);
     if ((uint64_t)n_states * (uint64_t)chunks > NA_SCRATCH_DOUBLES) {
         sv::set_last_error("sv_final_sample_noalloc: n_states x chunks = " +
                            std::to_string((uint64_t)n_states * chunks) + " partial sums exceed the static scratch of " +

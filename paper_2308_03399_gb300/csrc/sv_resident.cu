@@ -14,7 +14,7 @@ template <class R> size_t res_smem(const ResDesc& p) {
     const size_t warps = resident_threads(sizeof(R) == 8, p.np) / 32, mb = p.mb;
     return ((size_t)1 << p.np) * sizeof(typename Cplx<R>::T) + 2 * mb * p.block_words * 4 + mb * p.max_stages * 16 +
            (p.folds ? mb * (16 * FOLD_SPARSE + 8 * FOLD_LD) * 16 : 0) + mb * p.br_bytes + MAX_PEND * 8 +
-           warps * MAX_RED * 8 + RES_MAX_FINAL_CHUNKS * 8 + MAX_PEND * 4 + (((size_t)p.n_rows + 15) & ~(size_t)15);
+           warps * MAX_RED * 8 + RES_FINAL_BLOCKS * 8 + MAX_PEND * 4 + (((size_t)p.n_rows + 15) & ~(size_t)15);
 }
 
 const void* res_fn(int prec, int folds, int threads) {

@@ -95,8 +95,6 @@ template <class A> __device__ __forceinline__ A warp_total(A a) {
 }
 __device__ __forceinline__ float2 acc_pair(const Acc<float>& a) { return make_float2(a.hi, a.lo); }
 __device__ __forceinline__ double acc_pair(const Acc<double>& a) { return a.s; }
-__device__ __forceinline__ float2 sum_pair(const svs::Sum<float>& a) { return make_float2(a.hi, a.lo); }
-__device__ __forceinline__ double sum_pair(const svs::Sum<double>& a) { return a.s; }
 
 // Diagonal forms: |v|^2 of a group's amplitudes into the bins of the reduced
 // qubits (group bit 0, or bits 0 and 1).  A register pass over w qubits adds
@@ -248,6 +246,20 @@ __device__ __forceinline__ void res_dense(float2* st, const float4* M, const int
     }
 }
 
+// the sums of the 256-amplitude blocks of a chunk but for its last, from the
+// state in shared memory: this warp's w, w + step, ...  (complex128 states are
+// searched without them)
+static __device__ __forceinline__ void res_block_sums(const float2* st, int j0, int len, double* blocks, int w, int step) {
+    for (int k = w; k < len / 256 - 1; k += step) {
+        const double t = svs::block_sum([&](int j) {
+            const float2 x = st[swz(j0 + 256 * k + j)], y = st[swz(j0 + 256 * k + j + 1)];
+            return make_float4(x.x, x.y, y.x, y.y);
+        });
+        if ((threadIdx.x & 31) == 0) blocks[k] = t;
+    }
+}
+static __device__ __forceinline__ void res_block_sums(const double2*, int, int, double*, int, int) {}
+
 template <class R, int NT, bool FOLDS>
 __global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resident(DevBatch d, const __grid_constant__ ResDesc p) {
     using T = typename Cplx<R>::T;
@@ -267,8 +279,9 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resi
     unsigned char* const brm = reinterpret_cast<unsigned char*>(works + (p.folds ? mb * 8 * FOLD_LD : 0));
     double* const scale_col = reinterpret_cast<double*>(brm + mb * p.br_bytes);
     A* const redw = reinterpret_cast<A*>(scale_col + MAX_PEND);
-    double* const fin = reinterpret_cast<double*>(redw + nw * MAX_RED);
-    int32_t* const sel_col = reinterpret_cast<int32_t*>(fin + RES_MAX_FINAL_CHUNKS);
+    double* const fin = reinterpret_cast<double*>(redw);  // at most 8 chunk sums, after the last pass (none of a lone chunk)
+    double* const blocks = reinterpret_cast<double*>(redw + nw * MAX_RED);
+    int32_t* const sel_col = reinterpret_cast<int32_t*>(blocks + RES_FINAL_BLOCKS);
     uint8_t* const rows = reinterpret_cast<uint8_t*>(sel_col + MAX_PEND);
     const int2* const index = reinterpret_cast<const int2*>(d.ipool + p.index_off);
     const int2* const batches = reinterpret_cast<const int2*>(d.ipool + p.batch_off);  // first block, blocks
@@ -685,32 +698,45 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resi
         }
         __syncthreads();
 
-        // the final state to its slot, and the final sample
+        // the final state to its slot, and the final sample: the chunks of
+        // every other final sample, summed in the order of chunk_sum_warp, and
+        // (complex64) the blocks that sample_warp may pass over in the draw's
+        // chunk
         T* const out = reinterpret_cast<T*>(d.states) + (int64_t)shot * d.dim;
         const int dim = (int)d.dim;
         for (int j = tid; j < dim; j += nth) out[j] = st[swz(j)];
         if (p.has_final) {
-            const int len = dim < 256 ? dim : 256, chunks = dim / len;
-            for (int c = warp; c < chunks; c += nw) {
+            const int chunks = svs::final_chunks(dim), len = dim / chunks;
+            const double u = philox_uniform(d.seed, gs, p.fin_op);
+            constexpr int PER = sizeof(R) == 4 ? 2 : 1;  // neighbouring amplitudes of a lane
+            for (int c = warp; chunks > 1 && c < chunks; c += nw) {
                 svs::Sum<R> a;
+#pragma unroll 2
+                for (int j = PER * lane; j < len; j += 32 * PER)
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int j = lane * 8 + e;
-                    if (j < len) {
-                        const T x = st[swz(c * len + j)];
+                    for (int e = 0; e < PER; ++e) {
+                        const T x = st[swz(c * len + j + e)];
                         a.add_sq(x.x, x.y);
                     }
-                }
-                const A t = warp_total(sum_pair(a));
-                if (lane == 0) fin[c] = acc_get(t);
+                const double t = svs::warp_sum(a.wide());
+                if (lane == 0) fin[c] = t;
             }
+            if (chunks > 1) {
+                __syncthreads();
+                if (warp == 0) {
+                    svs::chunk_cum(fin, fin, chunks, 1);
+                    __syncwarp();
+                    const unsigned m = __ballot_sync(0xffffffffu, lane < chunks && u < fin[lane]);
+                    if (lane == 0) n_act[0] = m ? __ffs(m) - 1 : 0;  // the draw's chunk
+                }
+                __syncthreads();
+            }
+            res_block_sums(st, chunks > 1 ? n_act[0] * len : 0, len, blocks, warp, nw);
             __syncthreads();
             if (warp == 0) {
-                svs::chunk_cum(fin, fin, chunks, 1);
-                __syncwarp();
-                const double u = philox_uniform(d.seed, gs, p.fin_op);
                 double lo, hi;
-                const int64_t key = svs::sample_warp<R>(out, dim, chunks, fin, 1, u, &lo, &hi);
+                const int64_t key =
+                    svs::sample_warp<R, sizeof(R) == 4>(out, dim, chunks, fin, 1, u, &lo, &hi, blocks);
                 if (lane == 0) d.keys[shot] = (uint64_t)key;
             }
         }

@@ -9,7 +9,7 @@
 namespace sv {
 
 constexpr int RES_MAX_BATCH = 8;              // blocks prepared side by side
-constexpr int RES_MAX_FINAL_CHUNKS = 64;      // 2^14 amplitudes in chunks of 256
+constexpr int RES_FINAL_BLOCKS = 8;           // of 256 amplitudes in a chunk of the final sample
 constexpr int RES_MAX_ROWS = 8192;            // Pauli ops of a resident run (one byte each)
 constexpr size_t RES_MAX_SMEM = 224 * 1024;   // dynamic shared memory of a CTA
 

@@ -2327,7 +2327,7 @@ sv_status sv_alloc_batch(int n_qubits, uint64_t n_shots, int n_clbits, sv_prec p
     b->max_active = DEFAULT_MAX_ACTIVE;
     const int64_t tiles = 1ll << (n_qubits - b->tb);
     b->chunks = (int)std::min<int64_t>(tiles, MAX_CHUNKS);
-    b->chunks_final = (int)std::min<int64_t>(std::max<int64_t>(b->dim / 2048, 1), MAX_FINAL_CHUNKS);
+    b->chunks_final = svs::final_chunks(b->dim);
     if (cuda_stream) {
         b->stream = (cudaStream_t)cuda_stream;
     } else {

@@ -1,12 +1,13 @@
 // Philox draws and the final sampling building blocks (Section IV-B-2's
 // sampling measure), used by
-// the batch path (sv_kernels.cu) and by sv_final_sample_noalloc
-// (sv_noalloc.cu), so both give the same key for the same state and draw.
+// the batch path (sv_kernels.cu), resident runs (sv_resident.cuh) and
+// sv_final_sample_noalloc (sv_noalloc.cu), so all give the same key for the
+// same state and draw.
 //
 // A state of 2^n amplitudes is cut into `chunks` contiguous chunks of L
-// amplitudes.  chunk_sum() / chunk_sum_warp() give one chunk's sum of
-// |psi_j|^2 (one CTA or one warp, float-float or float64 per lane, the lanes
-// combined to float64 precision in a fixed order); chunk_cum()
+// amplitudes (final_chunks).  chunk_sum() / chunk_sum_warp() give one chunk's
+// sum of |psi_j|^2 (one CTA or one warp, float-float or float64 per lane, the
+// lanes combined to float64 precision in a fixed order); chunk_cum()
 // turns a state's chunk sums into a running sum (one warp, fixed order);
 // sample_warp() draws one key: the chunk by a two-level warp search over the
 // running sums, then the first j with u < C_j by a warp prefix sum over 256
@@ -44,6 +45,13 @@ __device__ __forceinline__ uint64_t philox_k53(uint64_t seed, uint64_t shot, uin
 // the uniform draw u = k * 2^-53 in [0, 1)
 __device__ __forceinline__ double philox_uniform(uint64_t seed, uint64_t shot, uint32_t op) {
     return (double)philox_k53(seed, shot, op) * 0x1.0p-53;
+}
+
+// chunks of a state's final sample: 2048 amplitudes each, at most 1024 of them
+constexpr int64_t CHUNK_AMPS = 2048;
+__host__ __device__ __forceinline__ int final_chunks(int64_t dim) {
+    const int64_t c = dim / CHUNK_AMPS;
+    return (int)(c < 1 ? 1 : (c > 1024 ? 1024 : c));
 }
 
 template <class R> struct Cx;
@@ -116,6 +124,22 @@ template <> struct Sum<float> {
     }
     __device__ __forceinline__ Sum3 wide() const { return {hi, lo, 0.f}; }
 };
+// the sum of |psi_j|^2 over 256 amplitudes, one warp, every lane; pair(j)
+// gives amplitudes j and j + 1 (j even)
+template <class Pair> __device__ __forceinline__ double block_sum(Pair pair) {
+    float4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = pair(2 * ((threadIdx.x & 31) + 32 * k));
+    Sum3 t;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        t.add_sq(v[k].x);
+        t.add_sq(v[k].y);
+        t.add_sq(v[k].z);
+        t.add_sq(v[k].w);
+    }
+    return warp_sum(t);
+}
 
 // amplitudes j and j + 1 (j even): one 128-bit load where the state starts on
 // a 16-byte boundary
@@ -222,17 +246,19 @@ __device__ __forceinline__ void chunk_cum(const double* sums, double* cum, int c
     }
 }
 
-// one key for draw u from the state g (whole warp; result in every lane)
-template <class R>
+// one key for draw u from the state g (whole warp; result in every lane);
+// BLOCKS: the caller has the block_sums of the draw's chunk, but for its last
+template <class R, bool BLOCKS = false>
 __device__ __forceinline__ int64_t sample_warp(const typename Cx<R>::T* g, int64_t dim, int chunks,
                                                const double* cum, int stride, double u, double* lo_out,
-                                               double* hi_out) {
+                                               double* hi_out, const double* blocks = nullptr) {
     using T = typename Cx<R>::T;
     const int lane = threadIdx.x & 31;
     const int64_t L = dim / chunks;
-    // chunk: first c with u < cum[c], coarse blocks of 32 then within
-    int c = chunks;
-    {
+    // chunk: first c with u < cum[c], coarse blocks of 32 then within; a
+    // lone chunk is searched as it is
+    int c = chunks > 1 ? chunks : 0;
+    if (chunks > 1) {
         const int nb = (chunks + 31) / 32;
         int blk = nb;
         for (int b0 = 0; b0 < nb && blk == nb; b0 += 32) {
@@ -260,20 +286,14 @@ __device__ __forceinline__ int64_t sample_warp(const typename Cx<R>::T* g, int64
                 // float64 takes 45 of 16 clocks); the running sums below
                 // only for the block that holds the draw
                 if (L > 256) {
-                    const typename Cx<R>::T* gb = g + j0 + blk;
-                    const bool aligned = (reinterpret_cast<uintptr_t>(gb) & 15) == 0;
-                    float4 v[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) v[k] = load_pair(gb + 2 * (lane + 32 * k), aligned);
-                    Sum3 t;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        t.add_sq(v[k].x);
-                        t.add_sq(v[k].y);
-                        t.add_sq(v[k].z);
-                        t.add_sq(v[k].w);
+                    double tot;
+                    if constexpr (BLOCKS) {
+                        tot = blk + 256 < L ? blocks[blk / 256] : 0.0;
+                    } else {
+                        const typename Cx<R>::T* gb = g + j0 + blk;
+                        const bool aligned = (reinterpret_cast<uintptr_t>(gb) & 15) == 0;
+                        tot = block_sum([&](int j) { return load_pair(gb + j, aligned); });
                     }
-                    const double tot = warp_sum(t);
                     if (!(u < acc + tot) && blk + 256 < L) {
                         acc += tot;
                         continue;
