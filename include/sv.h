@@ -246,9 +246,13 @@ sv_status sv_waiting(sv_batch b, uint64_t *n_waiting);
  * sv_get_keys.  use_graph != 0 captures the launch sequence into a CUDA
  * graph once per circuit and replays it.  Small registers (up to 14 qubits,
  * 13 in complex128) may run as one kernel with every shot's state in shared
- * memory, in shot-branching modes too when each shot has a state slot; the
- * results are the same.  SV_OPT_LOG, or a pass-shaping option away from its
- * default, keeps a run on the pass kernels.                                 */
+ * memory, in shot-branching modes too when each shot has a state slot.
+ * Choices and keys follow the same rules on both; the probabilities of Kraus
+ * ops and measurements are summed in another order there, so a choice can
+ * differ from the other form's only for a draw within about 1e-14 of a
+ * threshold, and a complex64 state by one float32 rounding per such op.
+ * SV_OPT_LOG, or an explicit value of a pass-shaping option (0 leaves it to
+ * the library), keeps a run on the pass kernels.                            */
 sv_status sv_run_circuit(sv_batch b, const sv_circuit *c, int use_graph);
 
 /* Several circuits, one per batch (n of them, batches sharing one stream;

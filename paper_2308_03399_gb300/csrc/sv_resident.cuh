@@ -13,7 +13,12 @@
 // of blocks in the integer pool (sv_resident.h).  Every amplitude goes
 // through the arithmetic of the register pass kernel in the same order
 // (stage by stage, or the folded matrix where the pass was folded), so
-// complex64 states are the same to the last bit.
+// without Kraus ops and measurements complex64 states are the same to the
+// last bit.  The probabilities of those are sums over the whole state, here
+// over other lanes than in a pass (float-float per lane, float64 across
+// lanes and warps in both): they agree to about 1e-14, and the factor
+// 1 / sqrt(p) of a choice, rounded to float32, can come out one float32
+// rounding apart (some 1e-7 of the choices).
 //
 // The stage code is kept small on purpose: CTAs sit in different stages, so
 // the instruction cache sees all of it at once.  (A first version that held
@@ -74,27 +79,35 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// float-float sum of two pairs (TwoSum of the high words, renormalised)
-__device__ __forceinline__ float2 ff_add(float2 a, float2 b) {
-    const float s = __fadd_rn(a.x, b.x);
-    const float bp = __fsub_rn(s, a.x);
-    float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bp)), __fsub_rn(b.x, bp));
-    e = __fadd_rn(e, __fadd_rn(a.y, b.y));
-    const float hi = __fadd_rn(s, e);
-    return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, s)));
+// a lane's accumulator as a value that the warp sums to float64 precision
+__device__ __forceinline__ svs::Sum3 wide(const Acc<float>& a) { return {a.hi, a.lo, 0.f}; }
+__device__ __forceinline__ double wide(const Acc<double>& a) { return a.s; }
+__device__ __forceinline__ svs::Sum3 pick(bool c, const svs::Sum3& a, const svs::Sum3& b) {
+    return {c ? a.hi : b.hi, c ? a.mid : b.mid, c ? a.lo : b.lo};
 }
-__device__ __forceinline__ double ff_add(double a, double b) { return a + b; }
-__device__ __forceinline__ float2 shfl_xor2(float2 a, int o) {
-    return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
-}
-__device__ __forceinline__ double shfl_xor2(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-template <class A> __device__ __forceinline__ A warp_total(A a) {
+__device__ __forceinline__ double pick(bool c, double a, double b) { return c ? a : b; }
+
+// Totals over the warp of four accumulators, to float64 precision as in the
+// register passes: total r comes out in the lanes with lane >> 3 == r.  The
+// lanes share the values out before they add, 6 merges for all four where a
+// tree for each takes 20 (12-qubit QFT with Kraus noise x 4000: 17.0 ms, and
+// 18.0 with float64 adds shared out in the same way).
+template <class R>
+__device__ __forceinline__ double warp_totals(const Acc<R>& a0, const Acc<R>& a1, const Acc<R>& a2, const Acc<R>& a3) {
+    using svs::lane_xor;
+    using svs::merge;
+    const int lane = threadIdx.x & 31;
+    const bool h = lane & 16, l = lane & 8;
+    auto w0 = wide(a0), w1 = wide(a1), w2 = wide(a2), w3 = wide(a3);
+    auto x = pick(h, w2, w0), y = pick(h, w3, w1);
+    merge(x, lane_xor(pick(h, w0, w2), 16));
+    merge(y, lane_xor(pick(h, w1, w3), 16));
+    auto t = pick(l, y, x);
+    merge(t, lane_xor(pick(l, x, y), 8));
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a = ff_add(a, shfl_xor2(a, o));
-    return a;
+    for (int o = 4; o > 0; o >>= 1) merge(t, lane_xor(t, o));
+    return svs::value(t);
 }
-__device__ __forceinline__ float2 acc_pair(const Acc<float>& a) { return make_float2(a.hi, a.lo); }
-__device__ __forceinline__ double acc_pair(const Acc<double>& a) { return a.s; }
 
 // Diagonal forms: |v|^2 of a group's amplitudes into the bins of the reduced
 // qubits (group bit 0, or bits 0 and 1).  A register pass over w qubits adds
@@ -263,7 +276,6 @@ static __device__ __forceinline__ void res_block_sums(const double2*, int, int, 
 template <class R, int NT, bool FOLDS>
 __global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resident(DevBatch d, const __grid_constant__ ResDesc p) {
     using T = typename Cplx<R>::T;
-    using A = typename AccSlot<R>::T;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int n_act[RES_MAX_BATCH];  // active stages of a block; for a folded one, entries per row
     __shared__ unsigned long long clb_sh, hist_sh;
@@ -278,9 +290,9 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resi
     float4* const works = tabs + (p.folds ? mb * 16 * FOLD_SPARSE : 0);
     unsigned char* const brm = reinterpret_cast<unsigned char*>(works + (p.folds ? mb * 8 * FOLD_LD : 0));
     double* const scale_col = reinterpret_cast<double*>(brm + mb * p.br_bytes);
-    A* const redw = reinterpret_cast<A*>(scale_col + MAX_PEND);
-    double* const fin = reinterpret_cast<double*>(redw);  // at most 8 chunk sums, after the last pass (none of a lone chunk)
-    double* const blocks = reinterpret_cast<double*>(redw + nw * MAX_RED);
+    double* const redw = scale_col + MAX_PEND;
+    double* const fin = redw;  // at most 8 chunk sums, after the last pass (none of a lone chunk)
+    double* const blocks = redw + nw * MAX_RED;
     int32_t* const sel_col = reinterpret_cast<int32_t*>(blocks + RES_FINAL_BLOCKS);
     uint8_t* const rows = reinterpret_cast<uint8_t*>(sel_col + MAX_PEND);
     const int2* const index = reinterpret_cast<const int2*>(d.ipool + p.index_off);
@@ -605,41 +617,54 @@ __global__ void __launch_bounds__(NT, (ResCta<R, NT, FOLDS>::min_blocks)) k_resi
             if (red) {
                 const int nv = red_kind == RED_DIAG ? 1 << red_k : red_R;  // values reduced over the state
                 if (red_kind == RED_BINS) {
-                    // a warp owns an outcome: its amplitudes, one compensated
-                    // addition each, in a fixed order
+                    // a warp owns up to four outcomes at a time: their
+                    // amplitudes, one compensated addition each, in a fixed
+                    // order
                     __syncthreads();
                     // (the measured qubits are group bits 0.. in order)
-                    for (int o = warp; o < red_R; o += nw) {
-                        Acc<R> a;
-                        a.zero();
-                        for (int m = o; m < 16; m += red_R) {
-                            const int om = off(m);
+                    for (int o0 = warp; o0 < red_R; o0 += 4 * nw) {
+                        Acc<R> a[4];
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) a[r].zero();
+                        for (int m = 0; m < 16; m += red_R) {
+                            int om[4];
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) om[r] = off((o0 + r * nw + m) & 15);
+                            if (o0 + nw >= red_R) {  // the warp's only outcome
 #pragma unroll 4
+                                for (int g = lane; g < groups; g += 32) {
+                                    const T x = st[group_base(g) ^ om[0]];
+                                    a[0].add(x.x * x.x + x.y * x.y);
+                                }
+                                continue;
+                            }
+#pragma unroll 2
                             for (int g = lane; g < groups; g += 32) {
-                                const T x = st[group_base(g) ^ om];
-                                a.add(x.x * x.x + x.y * x.y);
+                                const int base = group_base(g);
+#pragma unroll
+                                for (int r = 0; r < 4; ++r)
+                                    if (o0 + r * nw < red_R) {
+                                        const T x = st[base ^ om[r]];
+                                        a[r].add(x.x * x.x + x.y * x.y);
+                                    }
                             }
                         }
-                        const A t = warp_total(acc_pair(a));
-                        if (lane == 0) redw[o] = t;
+                        const double t = warp_totals<R>(a[0], a[1], a[2], a[3]);
+                        const int o = o0 + (lane >> 3) * nw;
+                        if ((lane & 7) == 0 && o < red_R) redw[o] = t;
                     }
                 } else {
-#pragma unroll
-                    for (int r = 0; r < REG_MAX_RED; ++r) {
-                        if (r >= nv) break;
-                        const A t = warp_total(acc_pair(acc[r]));
-                        if (lane == 0) redw[warp * MAX_RED + r] = t;
-                    }
+                    const double t = warp_totals<R>(acc[0], acc[1], acc[2], acc[3]);  // (zeros past nv)
+                    if ((lane & 7) == 0 && lane >> 3 < nv) redw[warp * MAX_RED + (lane >> 3)] = t;
                 }
                 __syncthreads();
                 if (warp == 0) {
                     // totals (lane r: value r), then the probabilities
                     double val = 0.0;
                     if (lane < nv) {
-                        A t = redw[lane];
+                        val = redw[lane];
                         if (red_kind != RED_BINS)
-                            for (int w = 1; w < nw; ++w) t = ff_add(t, redw[w * MAX_RED + lane]);
-                        val = acc_get(t);
+                            for (int w = 1; w < nw; ++w) val += redw[w * MAX_RED + lane];
                     }
                     double pr = val;
                     if (red_kind == RED_DIAG) {
