@@ -1718,62 +1718,93 @@ bool resident_candidate(sv_batch b) {
     return b->n <= (b->prec == SV_C128 ? RES_MAX_QUBITS_C128 : RES_MAX_QUBITS_C64);
 }
 
+// two back-to-back one-qubit Kraus ops that one pass and one decide take
+bool joint_pair(sv_batch b, const sv_circuit* c, int i) {
+    return b->joint && i + 1 < c->n_ops && c->kind[i] == SV_OP_KRAUS && c->kind[i + 1] == SV_OP_KRAUS &&
+           c->nq[i] == 1 && c->nq[i + 1] == 1 && c->qubits[c->q_off[i]] != c->qubits[c->q_off[i + 1]] &&
+           c->n_terms[i] * c->n_terms[i + 1] <= MAX_RED;
+}
+
+// probability of an op's likeliest outcome: from its table, or for Kraus ops
+// on the maximally mixed state.  Measured outcomes may be certain (a syndrome
+// of a code state), so a measurement is taken to leave the branches together.
+double likeliest(const sv_circuit* c, int i) {
+    const double* d = c->data + c->d_off[i];
+    double p = 0.0;
+    if (c->kind[i] == SV_OP_PAULI) {
+        for (int t = 0; t < c->n_terms[i]; ++t) p = std::max(p, d[t] - (t ? d[t - 1] : 0.0));
+    } else if (c->kind[i] == SV_OP_KRAUS) {
+        const int entries = 2 << (2 * c->nq[i]);
+        for (int t = 0; t < c->n_terms[i]; ++t) {
+            double w = 0.0;
+            for (int e = 0; e < entries; ++e) w += d[(size_t)t * entries + e] * d[(size_t)t * entries + e];
+            p = std::max(p, w / (1 << c->nq[i]));
+        }
+    } else {
+        p = 1.0;
+    }
+    return std::min(1.0, std::max(0.0, p));
+}
+
 // Shot-branching shares the states of shots that agree so far but pays a
 // decide, a copy and a pass launch per random op; a resident run simulates
-// every shot by itself in one launch (12-qubit SU(4) x 4000: 2.6 ms branching
-// and 3.8 ms resident at noise 1e-4, 4.2 and 3.8 ms at 3e-2; 12-qubit QFT x
-// 4000: 5.7 and 1.6 ms, 9.0 and 1.7 ms).  Both are estimated in microseconds
-// from GB300 timings (circuits of 6 to 13 qubits, 100 to 4000 shots,
-// noise of 1e-4 to 3e-2): the
-// branching run from its launches and the number of live branches that the
-// noise probabilities lead to expect, the resident run from the passes of
-// every shot.  It has to come out clearly ahead.
+// every shot by itself in one launch (12-qubit QFT with Kraus noise x 1000:
+// 17.3 ms branching and 4.7 ms resident; 14-qubit brickwork x 4000 at noise
+// 1e-4: 1.3 and 3.3 ms).  Both are estimated in microseconds from GB300
+// timings (ten families of 7 to 14 qubits, 100 to 10000 shots, noise of 1e-5
+// to 1e-2): the branching run from its decides, passes and live branches, the
+// resident run from the passes and stages of every shot.  It has to come out
+// clearly ahead: over those 811 runs in shot-branching mode none came out more
+// than 3% slower than on the pass kernels before resident runs.
 bool resident_pays(sv_batch b, const sv_circuit* c, const std::vector<Launch>& launches) {
-    const double S = (double)b->n_shots, dim = (double)b->dim;
+    const double S = (double)b->n_shots, dim = (double)b->dim, roots = std::max(1, b->n_psets);
     const bool c128 = b->prec == SV_C128;
-    // expected live branches, averaged over the random ops; decides in chains
-    double keep = 1.0, live = 0.0, roots = std::max(1, b->n_psets);
-    int ops = 0, chains = 0, tail = 0;
+    // decides, each with the ops that chain_decide lets it take along; live
+    // branches averaged over the random ops: the shots without an error, one
+    // branch per single error that some shot took, and a branch per shot of
+    // more errors
+    double errors = 0.0, singles = 0.0, live = 0.0;
+    int ops = 0, chains = 0, tail = 0, nk = 0;
     for (int i = 0; i < c->n_ops; ++i) {
-        const int kind = c->kind[i], k = c->nq[i];
-        const double* d = c->data + c->d_off[i];
-        double p0 = 1.0;  // probability of the likeliest outcome
-        if (kind == SV_OP_PAULI) {
-            p0 = d[0];
-        } else if (kind == SV_OP_KRAUS) {
-            p0 = 0.0;
-            for (int t = 0; t < c->n_terms[i]; ++t) {
-                double w = 0.0;
-                for (int e = 0; e < 2 << (2 * k); ++e) w += d[(size_t)t * (2 << (2 * k)) + e] * d[(size_t)t * (2 << (2 * k)) + e];
-                p0 = std::max(p0, w / (1 << k));
-            }
-        } else if (kind == SV_OP_MEASURE) {
-            p0 = 1.0 / (1 << k);
+        const int kind = c->kind[i];
+        if (kind != SV_OP_PAULI && kind != SV_OP_KRAUS && kind != SV_OP_MEASURE) continue;
+        const bool pair = joint_pair(b, c, i);
+        const int R = kind == SV_OP_MEASURE ? 1 << c->nq[i] : c->n_terms[i];
+        if (kind == SV_OP_PAULI && chains && tail < MAX_TAIL && nk * R <= MAX_TERMS) {
+            ++tail;
+            nk *= R;
         } else {
-            if (kind == SV_OP_GATE && k > 2) tail = 0;
-            continue;
-        }
-        keep *= std::min(1.0, std::max(0.0, p0));
-        ++ops;
-        live += std::min(S, roots + S * (1.0 - keep));
-        // Pauli ops follow a decide as its tail, up to MAX_TAIL of them
-        if (kind == SV_OP_PAULI && tail < MAX_TAIL && ops > 1) ++tail;
-        else {
             ++chains;
-            tail = 0;
+            tail = pair ? 1 : 0;
+            nk = pair ? R * c->n_terms[i + 1] : R;
         }
+        for (int j = i; j <= i + pair; ++j) {
+            errors -= std::log(std::max(likeliest(c, j), 1e-9));
+            if (kind != SV_OP_MEASURE) singles += c->n_terms[j] - 1;
+            const double p0 = std::exp(-errors), p1 = errors * p0, s = S / roots;
+            const double one = singles > 0 ? singles * (1.0 - std::exp(-s * p1 / singles)) : 0.0;
+            ++ops;
+            live += std::min(S, roots * (1.0 + one + s * (1.0 - p0 - p1)));
+        }
+        i += pair;
     }
     if (ops) live /= ops;
-    double passes = 0;
-    for (const Launch& L : launches) {
-        if (L.type != L_PASS) continue;
-        passes += 1;
-    }
-    const double branch = chains * (14.0 + 0.0037 * S) + passes * (8.0 + std::min(dim, 8192.0) * (c128 ? 8e-3 : 4.3e-3)) +
-                          passes * live * (double)b->state_bytes * 2.0 / 3.5e6;
-    // per pass a latency floor, and nanoseconds of the chip per state
-    const double resident = c128 ? passes * std::max(12.0 + dim * 0.016, S * (35.0 + dim * 0.09) * 1e-3)
-                                 : passes * std::max(8.5, S * (6.0 + dim * 0.0026) * 1e-3);
+    double passes = 0, stages = 0;
+    for (const Launch& L : launches)
+        if (L.type == L_PASS) {
+            passes += 1;
+            stages += L.pass.n_stages;
+        }
+    // (a pass's launch and its work on one branch; then every live one's bytes)
+    const double branch =
+        (c128 ? chains * (14.0 + 3.7e-3 * S) + passes * (8.0 + 8e-3 * std::min(dim, 8192.0))
+              : chains * (18.0 + 1.25e-3 * S) + passes * (10.0 + 3e-3 * std::min(dim, 8192.0))) +
+        passes * live * (double)b->state_bytes * 2.0 / 3.5e6;
+    // a latency floor per pass, and the chip's time per state: passes, stages
+    // and the final sample
+    const double resident =
+        c128 ? passes * std::max(10.0 + 0.014 * dim, S * (35.0 + 0.09 * dim) * 1e-3)
+             : std::max(passes * 8.5, S * 1e-3 * (passes * (1.9 + 2.1e-3 * dim) + 0.136 * stages + 19.4 + 0.016 * dim));
     return resident < 0.8 * branch;
 }
 
@@ -2219,9 +2250,7 @@ sv_status record_ops(sv_batch b, const sv_circuit* c, std::vector<Launch>& launc
     b->term_count_i.clear();
     launches.clear();
     for (int i = 0; i < c->n_ops && !st; ++i) {
-        if (b->joint && i + 1 < c->n_ops && c->kind[i] == SV_OP_KRAUS && c->kind[i + 1] == SV_OP_KRAUS &&
-            c->nq[i] == 1 && c->nq[i + 1] == 1 && c->qubits[c->q_off[i]] != c->qubits[c->q_off[i + 1]] &&
-            c->n_terms[i] * c->n_terms[i + 1] <= MAX_RED) {
+        if (joint_pair(b, c, i)) {
             st = op_kraus_pair(b, (uint32_t)i, c->qubits[c->q_off[i]], c->n_terms[i], c->data + c->d_off[i],
                                (uint32_t)(i + 1), c->qubits[c->q_off[i + 1]], c->n_terms[i + 1],
                                c->data + c->d_off[i + 1]);
