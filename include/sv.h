@@ -317,7 +317,12 @@ sv_status sv_get_branch_tree(sv_batch b, int64_t *records, uint64_t cap, uint64_
  * doubles): live branches, waiting shots, kernel launches issued, passes,
  * algorithmic bytes of the pass kernels (each live state read once, and
  * written once when the pass applies ops), bytes of fork copies, waiting-
- * list restarts, bytes copied host to device.  Synchronises.               */
+ * list restarts, bytes copied host to device.  Synchronises.
+ * After a shot-branching run that ran as one kernel (see sv_run_circuit; one
+ * launch, a state per shot) the live branches are the shots with different
+ * outcomes, as forking would have left them, and the fork copies are those
+ * that forking would have made: that run itself copies no state, and its
+ * passes add one write of every shot's state to the bytes.                  */
 sv_status sv_stats(sv_batch b, double *stats);
 
 /* With SV_OPT_PROFILE: milliseconds spent per launch class (8 doubles:

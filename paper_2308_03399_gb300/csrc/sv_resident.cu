@@ -23,7 +23,33 @@ const void* res_fn(int prec, int folds, int threads) {
     return threads > 128 ? (const void*)k_resident<float, 512, true> : (const void*)k_resident<float, 128, true>;
 }
 
+// open addressing, at most half full; 0 marks a free slot
+__global__ void k_history_count(const unsigned long long* hist, uint64_t n, unsigned long long* tab, uint64_t mask,
+                                unsigned long long runs) {
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const unsigned long long h = hist[i] ? hist[i] : 1ull;
+    for (uint64_t k = 0; k <= mask; ++k) {
+        const unsigned long long old = atomicCAS(tab + HIST_COUNTS + ((h + k) & mask), 0ull, h);
+        if (old == h) return;
+        if (old == 0) {
+            atomicAdd(tab, runs);
+            atomicAdd(tab + 1, 1ull);
+            return;
+        }
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_history_count(const unsigned long long* hist, uint64_t n, unsigned long long* tab,
+                                 unsigned long long runs, cudaStream_t s) {
+    const size_t slots = history_slots(n);
+    cudaError_t e = cudaMemsetAsync(tab + 1, 0, 8 * (HIST_COUNTS - 1 + slots), s);
+    if (e != cudaSuccess) return e;
+    k_history_count<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(hist, n, tab, slots - 1, runs);
+    return cudaGetLastError();
+}
 
 // Warps of a CTA and blocks prepared side by side: a warp per 32 groups of 16
 // amplitudes while several CTAs fit an SM (their number, not the width of

@@ -70,6 +70,16 @@ int resident_threads(int prec, int np);
 inline bool resident_one_cta(int prec, int np) { return np >= (prec ? 13 : 14); }  // per SM
 int resident_batch(int prec, int np);  // most blocks of a batch
 size_t resident_smem_bytes(int prec, const ResDesc& p);
+// counts the different words of hist[0..n): words 1 and 0 of the table take
+// their number and the sum of number x runs; history_slots words follow
+constexpr int HIST_COUNTS = 2;
+inline size_t history_slots(uint64_t n) {
+    size_t s = 64;
+    while (s < 2 * n) s *= 2;
+    return s;
+}
+cudaError_t launch_history_count(const unsigned long long* hist, uint64_t n, unsigned long long* tab,
+                                 unsigned long long runs, cudaStream_t s);
 cudaError_t init_resident();
 cudaError_t launch_resident(const DevBatch& d, int prec, const ResDesc& p, int n_states, int n_sm, cudaStream_t s);
 

@@ -215,10 +215,13 @@ struct sv_batch_s {
     std::vector<Launch> res_list;
     uint64_t res_hash = 0, res_gen = 0;
     double res_bytes = 0;  // states written by resident runs since sv_stats
-    // resident runs of a shot-branching batch: a history word per shot, runs
-    // since sv_stats, and whether the last run was one
-    unsigned long long* d_hist = nullptr;
-    int64_t res_branch_runs = 0;
+    // resident runs of a shot-branching batch: a history word per shot and the
+    // table that counts the different ones (see fold_histories); the runs of
+    // the circuit res_key whose histories are not counted yet, the roots of
+    // those that are, and whether the last run was a resident one
+    unsigned long long *d_hist = nullptr, *d_hist_tab = nullptr;
+    uint64_t res_key = 0;
+    int64_t res_runs = 0, res_roots = 0;
     bool res_branch_last = false;
     std::map<int, int> term_count, term_count_i;  // terms at a pool / integer-pool offset (recording)
     // parameter sweep (sv_set_param_sets): every shot's parameter set
@@ -329,7 +332,6 @@ void count_launch(sv_batch b, const Launch& L) {
         b->pass_store.push_back(L.pass.store ? 1 : 0);
     } else if (L.type == L_RESIDENT) {
         b->n_passes += L.a0;
-        b->res_branch_runs += b->branch;
         b->res_bytes += (double)L.a1 * (double)b->state_bytes;
     }
 }
@@ -902,6 +904,7 @@ sv_status ensure_started(sv_batch b) {
     if (!b->rec) {  // per-op calls: a new run, a new fork log
         sv_status st = tree_begin(b);
         if (st) return st;
+        b->res_branch_last = false;
     }
     const int branch = b->branch;
     Launch r;
@@ -2206,8 +2209,10 @@ bool build_resident(sv_batch b, std::vector<Launch>& launches) {
         b->ipool.resize(ipool0);
         return false;
     }
-    if (b->branch) {  // sv_stats counts the histories (see there)
-        if (!b->d_hist && dalloc(b, &b->d_hist, b->n_shots) != SV_OK) {
+    if (b->branch) {  // sv_stats counts the histories
+        if (!b->d_hist_tab &&
+            (dalloc(b, &b->d_hist, b->n_shots) || dalloc(b, &b->d_hist_tab, HIST_COUNTS + history_slots(b->n_shots)) ||
+             cudaMemsetAsync(b->d_hist_tab, 0, 8 * HIST_COUNTS, b->stream) != cudaSuccess)) {
             b->ipool.resize(ipool0);
             return false;
         }
@@ -2233,6 +2238,36 @@ bool build_resident(sv_batch b, std::vector<Launch>& launches) {
     L.res = r;
     launches.assign(1, L);
     return true;
+}
+
+// A resident run of a shot-branching batch gives every shot a state of its
+// own; the branches it stands for are the different histories.  Runs of one
+// circuit leave the same words, so they are counted once for all of them:
+// when another circuit is about to overwrite them, or by sv_stats.
+sv_status fold_histories(sv_batch b) {
+    if (!b->res_runs) return SV_OK;
+    CU(launch_history_count(b->d_hist, b->n_shots, b->d_hist_tab, (unsigned long long)b->res_runs, b->stream));
+    int64_t roots = 1;
+    if (b->n_psets > 0) {
+        std::vector<uint32_t> ps(b->h_pset);
+        std::sort(ps.begin(), ps.end());
+        roots = std::unique(ps.begin(), ps.end()) - ps.begin();
+    }
+    b->res_roots += b->res_runs * roots;
+    b->res_runs = 0;
+    return SV_OK;
+}
+
+// a run of the circuit with this hash starts
+sv_status note_run(sv_batch b, uint64_t hash, bool resident) {
+    b->res_branch_last = b->branch && resident;
+    if (!b->res_branch_last) return SV_OK;
+    const uint64_t key = fnv(hash, &b->pool_gen, 8);
+    if (key != b->res_key)
+        if (sv_status st = fold_histories(b)) return st;
+    b->res_key = key;
+    b->res_runs += 1;
+    return SV_OK;
 }
 
 // the circuit is one resident launch (which starts from |0...0> by itself)
@@ -2605,6 +2640,7 @@ sv_status sv_set_param_sets(sv_batch b, const uint32_t* set_of_shot, uint32_t n_
     if (!b) return fail(SV_EINVAL, "batch is NULL");
     if (!b->pend.empty() || b->uncommitted || b->started)
         return fail(SV_EINVAL, "set the parameter sets before the first op of a run");
+    if (sv_status hs = fold_histories(b)) return hs;  // of runs with the sets so far
     if (n_sets == 0) {
         b->n_psets = 0;
         b->h_pset.clear();
@@ -2755,7 +2791,7 @@ sv_status sv_run_circuit(sv_batch b, const sv_circuit* c, int use_graph) {
         if ((st = upload_pool(b))) return st;
     }
     const int branch = b->branch && !resident;
-    b->res_branch_last = b->branch && resident;
+    if ((st = note_run(b, h, resident))) return st;
     int from_wait = 0;
     int n_run = (int)b->n_shots;
     if ((st = tree_begin(b))) return st;
@@ -2929,7 +2965,7 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
     for (int i = 0; i < n; ++i) {
         const bool resident = b0->multi_lists[i].back().type == L_RESIDENT;
         forks[i] = bs[i]->branch && !resident;
-        bs[i]->res_branch_last = bs[i]->branch && resident;
+        if ((st = note_run(bs[i], circuit_hash(bs[i], cs[i]), resident))) return st;
     }
     for (int i = 0; i < n; ++i)
         if ((st = tree_begin(bs[i]))) return st;
@@ -3300,24 +3336,18 @@ sv_status sv_stats(sv_batch b, double* s) {
     b->res_bytes = 0;
     for (int i = 0; i < np && i < (int)b->pass_store.size(); ++i)
         bytes += (double)nbr[i] * (double)b->state_bytes * (1.0 + b->pass_store[i]);
-    // a resident run of a shot-branching batch gave every shot a state of its
-    // own; the branches it stands for are the different histories
+    // resident runs of a shot-branching batch: see fold_histories
     double live = ctl[CTL_NBR], copied = ctl[CTL_NCOPIED];
-    if (b->res_branch_last && b->d_hist) {
-        std::vector<unsigned long long> h(b->n_shots);
-        CU(cudaMemcpyAsync(h.data(), b->d_hist, 8 * b->n_shots, cudaMemcpyDeviceToHost, b->stream));
+    if (b->d_hist_tab) {
+        if (sv_status st = fold_histories(b)) return st;
+        unsigned long long cnt[HIST_COUNTS];
+        CU(cudaMemcpyAsync(cnt, b->d_hist_tab, sizeof(cnt), cudaMemcpyDeviceToHost, b->stream));
+        CU(cudaMemsetAsync(b->d_hist_tab, 0, 8, b->stream));
         CU(cudaStreamSynchronize(b->stream));
-        std::sort(h.begin(), h.end());
-        live = (double)(std::unique(h.begin(), h.end()) - h.begin());
-        double roots = 1;
-        if (b->n_psets > 0) {
-            std::vector<uint32_t> ps(b->h_pset);
-            std::sort(ps.begin(), ps.end());
-            roots = (double)(std::unique(ps.begin(), ps.end()) - ps.begin());
-        }
-        copied += (double)b->res_branch_runs * (live - roots);
+        if (b->res_branch_last) live = (double)cnt[1];
+        copied += (double)cnt[0] - (double)b->res_roots;
+        b->res_roots = 0;
     }
-    b->res_branch_runs = 0;
     s[0] = live;
     s[1] = ctl[CTL_NWAIT];
     s[2] = (double)b->n_launch;
