@@ -1520,9 +1520,13 @@ uint64_t circuit_hash(sv_batch b, const sv_circuit* c) {
     h = fnv(h, c->d_off, 8 * n);
     h = fnv(h, c->cond_clbit, 4 * n);
     h = fnv(h, c->cond_val, 4 * n);
-    h = fnv(h, c->reset, 4 * n);
+    // (arrays that only measurements have may be NULL without one; what
+    // op_measure refuses is not read)
     for (size_t i = 0; i < n; ++i)
-        if (c->kind[i] == SV_OP_MEASURE) h = fnv(h, c->clbits + c->cl_off[i], 4 * (size_t)c->nq[i]);
+        if (c->kind[i] == SV_OP_MEASURE && c->nq[i] >= 1 && c->nq[i] <= 4 && c->clbits) {
+            h = fnv(h, c->clbits + c->cl_off[i], 4 * (size_t)c->nq[i]);
+            h = fnv(h, c->reset + i, 4);
+        }
     int64_t dmax = 0, qmax = 0;
     for (size_t i = 0; i < n; ++i) qmax = std::max<int64_t>(qmax, c->q_off[i] + c->nq[i]);
     h = fnv(h, c->qubits, 4 * qmax);
