@@ -16,11 +16,14 @@ constexpr int64_t REG_UNIT_MIN_AMPS = 8192;  // smallest register-path unit
 constexpr int PRE_WORDS = 8;                 // integer-pool words per pre-drawn Pauli row
 constexpr uint64_t PRE_TABLE_BYTES = 1ull << 30;  // largest pre-drawn Pauli table
 constexpr int MAX_RED = 16;        // probabilities reduced by one pass (Kraus terms, 2^m outcomes)
-// reduction partials per state: fine enough that the units of a few branches
+// reduction units per state: fine enough that the units of a few branches
 // of a large state still divide evenly over some 3000 warps (with 1024, three
-// 27-qubit branches left 98% of them idle in a second round: 4.2 TB/s)
+// 27-qubit branches left 98% of them idle in a second round: 4.2 TB/s).  A
+// state's sums are those of at most RED_CHUNKS chunks, each the sum of its
+// units in order: the same bits whether memory has room for a record per
+// unit or only per chunk.
 constexpr int MAX_CHUNKS = 8192;
-constexpr int MAX_FINAL_CHUNKS = 1024;  // chunks of the final sample
+constexpr int RED_CHUNKS = 1024;
 constexpr int MAX_STAGE_Q = 5;     // qubits of one stage (dense gates up to MAX_GATE_Q)
 constexpr int MAT_SMEM = 1024;     // complex matrix entries staged in shared memory per pass
 // fork log record: op, parent branch, child branch (-1: waiting list), outcome,
@@ -71,7 +74,8 @@ struct PassDesc {
     int32_t tile_q[MAX_TILE_BITS];
     int32_t n_nontile;
     int32_t nontile_q[32];
-    int32_t chunks;            // reduction chunks per state
+    int32_t chunks;            // units of work per state
+    int32_t sub;               // log2 of the units that share a reduction record
     int32_t tiles_per_chunk;
     int32_t n_stages;
     int32_t store;             // write the tile back
@@ -107,7 +111,8 @@ struct DecideDesc {
     int32_t kind;              // DEC_*
     int32_t R;                 // terms / outcomes
     int32_t pend;
-    int32_t chunks;            // partials to sum
+    int32_t chunks;            // chunks to sum
+    int32_t group;             // log2 of the records of a chunk
     int32_t fork;              // shot-branching on
     int32_t sample_only;       // draw and log the choices, change no branch (per-op
                                // calls in shot-branching mode: sv_branch commits)

@@ -672,14 +672,11 @@ struct DecTab {
     int leaf[MAX_TERMS];                  // fork log: branch of each outcome tuple
 };
 
-// probabilities of branch b into p_out (and, for Pauli, the table into
-// cum_out); one whole warp.  With joint_out (a DEC_KRAUS_J1 head), the
-// joint probabilities p_ij are kept there too.
 // where the terms of branch b's decide lie: the contiguous entries
-// [base, base + nk) of every chunk's record
+// [base, base + nk) of every record, 2^group records a chunk
 struct PartSrc {
     const double* pp;
-    int nk, inner;
+    int nk, inner, group;
 };
 __device__ __forceinline__ PartSrc part_src(const DevBatch& d, const DecideDesc& dd, int b, int slot) {
     int src = slot, base_r = 0, inner = 1;
@@ -692,7 +689,7 @@ __device__ __forceinline__ PartSrc part_src(const DevBatch& d, const DecideDesc&
         if (b >= cf && b < ce) src = d.br_slot[d.br_parent[b]];
         base_r = d.br_sel[(int64_t)dd.pend_prev * d.cap_br + b] * dd.R;  // p_ij = entry i * R + j
     }
-    return {d.partials + (int64_t)src * d.max_chunks * MAX_RED + base_r, dd.R * inner, inner};
+    return {d.partials + (int64_t)src * d.max_chunks * MAX_RED + base_r, dd.R * inner, inner, dd.group};
 }
 
 // this warp's share of the sums of a branch's terms, into out[0..nk).  Lanes
@@ -708,8 +705,23 @@ __device__ __forceinline__ void part_sums(const PartSrc& ps, int chunks, int w, 
     double u = 0.0;
     if (k < ps.nk) {
         const double* q = ps.pp + k;
+        if (ps.group == 0) {
 #pragma unroll 4
-        for (int c = c0; c < chunks; c += per * nw) u += q[(int64_t)c * MAX_RED];
+            for (int c = c0; c < chunks; c += per * nw) u += q[(int64_t)c * MAX_RED];
+        } else {
+            constexpr int MAX_RECS = MAX_CHUNKS / RED_CHUNKS;
+            const int n = 1 << ps.group;
+            for (int c = c0; c < chunks; c += per * nw) {
+                const double* rec = q + (int64_t)c * n * MAX_RED;
+                double v[MAX_RECS];
+#pragma unroll
+                for (int i = 0; i < MAX_RECS; ++i) v[i] = i < n ? rec[i * MAX_RED] : 0.0;
+#pragma unroll
+                for (int i = 1; i < MAX_RECS; ++i)
+                    if (i < n) v[0] += v[i];
+                u += v[0];
+            }
+        }
     }
     // lanes of chunks past the last hold exact zeros: only the levels that
     // mix used lanes
@@ -721,7 +733,10 @@ __device__ __forceinline__ bool decide_in_cta(const DecideDesc& dd, int cnt) {
     return cnt > DEC_SMALL || (dd.kind != DEC_PAULI && dd.chunks > DEC_WARP_CHUNKS);
 }
 
-// pre: per warp of the CTA its share of the sums (part_sums), nullable
+// probabilities of branch b into p_out (and, for Pauli, the table into
+// cum_out); one whole warp.  With joint_out (a DEC_KRAUS_J1 head), the
+// joint probabilities p_ij are kept there too.  pre: per warp of the CTA its
+// share of the sums (part_sums), nullable.
 __device__ void warp_probs(const DevBatch& d, const DecideDesc& dd, int b, int slot, double* p_out, double* cum_out,
                            double* joint_out, const double (*pre)[MAX_RED], int npre) {
     const int lane = threadIdx.x & 31;

@@ -511,11 +511,13 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
     for (int j = 0; j < WP; ++j) stride[j] = 1 << p.tile_q[j];
     // units are 2^k per branch; a warp takes a contiguous range of them.
     // Without a reduction the units of a branch that fall to the warp are one
-    // run of groups; with one, each unit writes its own partial.
+    // run of groups; with one, each unit writes its own partial, or (sub) the
+    // 2^sub units of a chunk, all of one warp, add up in the chunk's record.
     const int cshift = __ffs(p.chunks) - 1;
     const int64_t units = (int64_t)n_br << cshift;
     const int64_t gw = (int64_t)blockIdx.x * nwarps + warp, tw = (int64_t)gridDim.x * nwarps;
-    const int64_t u0 = units * gw / tw, u1 = units * (gw + 1) / tw;
+    const int sub = p.sub;
+    const int64_t u0 = (units >> sub) * gw / tw << sub, u1 = (units >> sub) * (gw + 1) / tw << sub;
     const int64_t unit_groups = (d.dim >> WP) >> cshift;
     const bool red = p.red_kind != RED_NONE;
     T* const states = reinterpret_cast<T*>(d.states);
@@ -794,6 +796,10 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
                 }
             }
         }
+        auto put = [&](int r, double x) {
+            double* q = &d.partials[((int64_t)slot * d.max_chunks + (c >> sub)) * MAX_RED + r];
+            *q = c & ((1ll << sub) - 1) ? *q + x : x;
+        };
         if (red && p.red_kind == RED_DIAG) {
             // the unit's bins, then every form from them: lane f writes form f
             const int D = 1 << p.red_k;
@@ -806,7 +812,7 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
 #pragma unroll
                 for (int r = 0; r < 4; ++r)
                     if (r < D) part += diag_weight(W, p.red_R, p.red_k, lane, r) * bin[r];
-                d.partials[((int64_t)slot * d.max_chunks + c) * MAX_RED + lane] = part;
+                put(lane, part);
             }
         } else if (BINS) {
             for (int r = 0; r < (1 << p.red_k); ++r) {  // every outcome's bin
@@ -818,14 +824,14 @@ __global__ void __launch_bounds__(RegCta<R>::threads, RegCta<R>::min_blocks)
                     a.s = bins[r * 32 + lane];
                 }
                 const double x = unit_total(a);
-                if (lane == 0) d.partials[((int64_t)slot * d.max_chunks + c) * MAX_RED + r] = x;
+                if (lane == 0) put(r, x);
             }
         } else if (red) {
 #pragma unroll
             for (int r = 0; r < REG_MAX_RED; ++r) {
                 if (r >= p.red_R) break;
                 const double x = unit_total(acc[r]);
-                if (lane == 0) d.partials[((int64_t)slot * d.max_chunks + c) * MAX_RED + r] = x;
+                if (lane == 0) put(r, x);
             }
         }
     }

@@ -131,7 +131,8 @@ struct sv_batch_s {
     size_t amp_bytes = 8, state_bytes = 0;
     int n_slots = 0;
     int tb = 11, chunks = 1, chunks_final = 1;
-    int red_chunks = 1;  // chunk records written by the last pass with a reduction
+    int max_units = 1;   // reduction units of a state at most (register passes)
+    int red_chunks = 1, red_group = 0;  // chunks of the last reduction, log2 of the records of each
     int threads = 256, grid_pass = 0, grid_small = 0, n_sm = 0;
     int max_active = 8, max_stages = MAX_STAGES;  // max_active is set in sv_alloc_batch
     bool max_active_set = false;  // SV_OPT_MAX_ACTIVE given explicitly (a new tile size keeps it)
@@ -450,6 +451,7 @@ int pool_matrix(sv_batch b, const double* m, int k, double scale = 1.0) {
 constexpr int DEFAULT_MAX_ACTIVE = 4;
 
 bool whole_active(sv_batch b);
+int ilog2(int64_t v) { return 63 - __builtin_clzll((unsigned long long)v); }
 int local_pos(const int* tile_q, int tb, int q) {
     for (int i = 0; i < tb; ++i)
         if (tile_q[i] == q) return i;
@@ -624,6 +626,13 @@ sv_status emit_stages(sv_batch b, const std::vector<int>& idx, const RedSpec& re
                                                   : std::max<int64_t>(b->dim / b->chunks, REG_UNIT_MIN_AMPS);
         p.chunks = (int)std::max<int64_t>(1, b->dim / unit);
         p.tiles_per_chunk = 1;
+        // a record per unit where the table holds them, else per chunk
+        const int group = std::max(0, ilog2(p.chunks) - ilog2(RED_CHUNKS));
+        if (red.kind != RED_NONE) {
+            p.sub = p.chunks > b->dev.max_chunks ? group : 0;
+            b->red_chunks = p.chunks >> group;
+            b->red_group = group - p.sub;
+        }
     } else {
         // tile path: with a reduction, a chunk spans at least eight tiles (or
         // the whole state), so the fixed-order combination of its sums is
@@ -631,11 +640,15 @@ sv_status emit_stages(sv_batch b, const std::vector<int>& idx, const RedSpec& re
         // its own (eight a unit left an 18-qubit density matrix on 32 CTAs:
         // 227 us a pass)
         const int64_t tiles = 1ll << (b->n - p.tb);
-        const int64_t tpc = red.kind == RED_NONE ? 1 : std::max<int64_t>(tiles / b->chunks, std::min<int64_t>(tiles, 8));
+        const int64_t tpc = red.kind == RED_NONE ? 1 : std::max<int64_t>(tiles / std::min(b->chunks, RED_CHUNKS),
+                                                                        std::min<int64_t>(tiles, 8));
         p.chunks = (int)(tiles / tpc);
         p.tiles_per_chunk = (int)tpc;
+        if (red.kind != RED_NONE) {
+            b->red_chunks = p.chunks;
+            b->red_group = 0;
+        }
     }
-    if (red.kind != RED_NONE) b->red_chunks = p.chunks;
     int mat = 0;
     if ((int)ss.size() > MAX_STAGES) return fail(SV_EINTERNAL, "pass holds more stages than a pass descriptor");
     p.n_stages = (int)ss.size();
@@ -1013,6 +1026,7 @@ sv_status emit_decide(sv_batch b, uint32_t op, int kind, int R, const double* cu
     d.R = R;
     d.pend = pend;
     d.chunks = b->red_chunks;  // the pass just emitted wrote these
+    d.group = b->red_group;
     d.fork = b->branch;
     d.m = m;
     d.r2 = r2;
@@ -1621,20 +1635,24 @@ sv_status run_plain(sv_batch b, const sv_circuit* c) {
                     }
                     if ((st = upload_pool(b))) return st;
                     if ((st = emit_pass(b, red))) return st;
-                    std::vector<double> part(MAX_RED * b->red_chunks);
-                    CU(cudaMemcpyAsync(part.data(), b->dev.partials, sizeof(double) * MAX_RED * b->red_chunks,
+                    const int recs = 1 << b->red_group;  // of a chunk
+                    std::vector<double> part((size_t)MAX_RED * b->red_chunks * recs);
+                    CU(cudaMemcpyAsync(part.data(), b->dev.partials, sizeof(double) * part.size(),
                                        cudaMemcpyDeviceToHost, b->stream));
                     CU(cudaStreamSynchronize(b->stream));
-                    if (kind == SV_OP_KRAUS) {
+                    auto total = [&](int r) {
                         double s = 0;
-                        for (int ch = 0; ch < b->red_chunks; ++ch) s += part[ch * MAX_RED];
-                        p[t] = s;
-                    } else {
-                        for (int o = 0; o < R; ++o) {
-                            double s = 0;
-                            for (int ch = 0; ch < b->red_chunks; ++ch) s += part[ch * MAX_RED + o];
-                            p[o] = s;
+                        for (int ch = 0; ch < b->red_chunks; ++ch) {
+                            double c = 0;
+                            for (int i = 0; i < recs; ++i) c += part[(size_t)(ch * recs + i) * MAX_RED + r];
+                            s += c;
                         }
+                        return s;
+                    };
+                    if (kind == SV_OP_KRAUS) {
+                        p[t] = total(0);
+                    } else {
+                        for (int o = 0; o < R; ++o) p[o] = total(o);
                         break;
                     }
                 }
@@ -2422,16 +2440,15 @@ sv_status sv_alloc_batch(int n_qubits, uint64_t n_shots, int n_clbits, sv_prec p
         const size_t reserve = std::max<size_t>(1ull << 30, total_b / 50);
         budget = free_b > fixed + reserve ? free_b - fixed - reserve : 0;
     }
-    // the finer chunks only where their partials cost no slot
+    // a record per reduction unit only where the records cost no slot
     const uint64_t most = mode == SV_PLAIN ? 1 : n_shots;
-    auto slots_with = [&](int chunks) {
-        const size_t per_slot = b->state_bytes + (size_t)std::max(chunks, b->chunks_final) * MAX_RED * 8;
-        return std::min<uint64_t>(budget / per_slot, most);
+    b->max_units = std::max(b->chunks, b->chunks_final);
+    auto slots_with = [&](int records) {
+        return std::min<uint64_t>(budget / (b->state_bytes + (size_t)records * MAX_RED * 8), most);
     };
-    const int coarse = std::min(b->chunks, MAX_FINAL_CHUNKS);
-    if (slots_with(b->chunks) < slots_with(coarse)) b->chunks = coarse;
-    const int max_chunks = std::max(b->chunks, b->chunks_final);
-    uint64_t slots = slots_with(b->chunks);
+    const int few = std::min(b->max_units, RED_CHUNKS);
+    const int max_chunks = slots_with(b->max_units) < slots_with(few) ? few : b->max_units;
+    uint64_t slots = slots_with(max_chunks);
     if (slots == 0) {
         sv_free_batch(b);
         return fail(SV_ENOMEM, "not even one state fits the memory budget");
@@ -2589,7 +2606,7 @@ static sv_status set_option(sv_batch b, sv_option opt, int64_t v) {
         if (v && (v < 2 || v > MAX_TILE_BITS)) return fail(SV_EINVAL, "tile bits must be 2..12");
         if (b->started) return fail(SV_EINVAL, "set the tile size before the first op");
         b->tb = std::min<int>(b->n, v ? (int)v : (b->prec == SV_C128 ? 10 : 11));
-        b->chunks = (int)std::min<int64_t>(1ll << (b->n - b->tb), b->dev.max_chunks);
+        b->chunks = (int)std::min<int64_t>(1ll << (b->n - b->tb), b->max_units);
         if (!b->max_active_set) b->max_active = DEFAULT_MAX_ACTIVE;
         return SV_OK;
     case SV_OPT_MAX_ACTIVE:
