@@ -26,6 +26,9 @@ constexpr int MAX_CHUNKS = 8192;
 constexpr int RED_CHUNKS = 1024;
 constexpr int MAX_STAGE_Q = 5;     // qubits of one stage (dense gates up to MAX_GATE_Q)
 constexpr int MAT_SMEM = 1024;     // complex matrix entries staged in shared memory per pass
+// k_pass's static shared memory (4.5 KB: stage tables, nonzero columns of
+// sparse matrices, warp sums) and the 1 KB the system keeps for every CTA
+constexpr int PASS_FIXED_SMEM = 4608 + 1024;
 // fork log record: op, parent branch, child branch (-1: waiting list), outcome,
 // shots, first perm position of the group's shots at the fork, first perm
 // position and shots of the forking node

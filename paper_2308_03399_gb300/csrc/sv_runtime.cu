@@ -299,8 +299,8 @@ int pass_grid(sv_batch b, const PassDesc& p) {
     // k_pass is register-bound at 512 threads per SM (two CTAs of 256);
     // shared memory (tile ring + matrices + accumulators) may allow fewer
     const int threads = tile_threads(b, p);
-    const size_t smem = pass_smem_bytes(b->prec == SV_C128, p, threads) + 2048;
-    const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(512 / threads, (227 * 1024) / smem));
+    const size_t smem = pass_smem_bytes(b->prec == SV_C128, p, threads) + PASS_FIXED_SMEM;
+    const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(512 / threads, (228 * 1024) / smem));
     return b->n_sm * per_sm;
 }
 
