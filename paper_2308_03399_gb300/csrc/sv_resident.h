@@ -25,10 +25,9 @@ enum : int32_t {
     RB_DECIDE = 3,
     RB_SO = 4,       // swizzled offsets of the four group bits
     RB_SF = 8,       // swizzled offsets of the other address bits, 16 bits each, in lane order
-    RB_RPOS = 14,    // group bits of the reduced qubits, 4 bits each
-    RB_FOLD = 15,    // the stages are composed into one 16 x 16 matrix
-    RB_RUN = 16,     // RED_DIAG: amplitudes per bin that a register pass's group adds up first
-    RB_STAGES = 20,
+    RB_FOLD = 14,    // the stages are composed into one 16 x 16 matrix
+    RB_RUN = 15,     // RED_DIAG: amplitudes per bin that a register pass's group adds up first
+    RB_STAGES = 16,
     RS_WORDS = 8
 };
 // stage words: 0: kind | k << 4 | reset << 8 | pre-drawn << 9 |

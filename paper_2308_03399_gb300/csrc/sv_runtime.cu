@@ -1921,10 +1921,12 @@ bool res_block(sv_batch b, const PassDesc& p, int s0, int s1, const std::vector<
     int gq[4];
     std::vector<int> order;
     res_group(fixed, np, gq, order);
+    bool in_group = true;  // every qubit that a stage or the reduction names
     auto gbit = [&](int pos) {
         const int q = p.tile_q[pos];
         for (int j = 0; j < 4; ++j)
             if (gq[j] == q) return j;
+        in_group = false;
         return 0;
     };
     B.w.assign(RB_STAGES + RS_WORDS * (s1 - s0), 0);
@@ -2020,12 +2022,15 @@ bool res_block(sv_batch b, const PassDesc& p, int s0, int s1, const std::vector<
         memcpy(&B.w[RB_STAGES + RS_WORDS * (s - s0)], S, sizeof(S));
     }
     *br_bytes = br;
+    if (!in_group) return false;
     if (!dec) {
         B.align(4);
         return true;
     }
+    // the kernel reads the reduced qubits at group bits 0, 1, ...
+    for (int j = 0; j < p.red_k; ++j)
+        if (gbit(p.red_pos[j]) != j || !in_group) return false;
     B.w[RB_RED] = p.red_kind | p.red_k << 4 | p.red_R << 8;
-    for (int j = 0; j < p.red_k; ++j) B.w[RB_RPOS] |= gbit(p.red_pos[j]) << (4 * j);
     if (p.red_kind == RED_DIAG) {
         if (p.red_k > 2 || p.red_R > MAX_RED) return false;
         B.w[RB_RUN] = p.reg_wp > 0 ? 1 << (p.reg_wp - p.red_k) : 1;
