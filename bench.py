@@ -124,9 +124,10 @@ def pass_traffic(args, alg_bytes_per_launch):
         return None
     rec = dict(ln.split(None, 1) for ln in open(path).read().strip().splitlines())
     # the pass kernels' sources: the kernel file and the headers holding the
-    # register kernel and the shared device helpers, hashed in this order
+    # register kernel, the stage folding and the shared device helpers, hashed
+    # in this order
     h = hashlib.sha1()
-    for f in ("sv_kernels.cu", "sv_pass_reg.cuh", "sv_common.cuh"):
+    for f in ("sv_kernels.cu", "sv_pass_reg.cuh", "sv_fold.cuh", "sv_common.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2308_03399_gb300", "csrc", f), "rb").read())
     sha = h.hexdigest()
     if rec.get("source_sha1") != sha or rec.get("workload") != f"{args.workload}:{args.mode}:{args.prec}":
