@@ -264,10 +264,12 @@ __device__ __forceinline__ void res_dense(float2* st, const float4* M, const int
 // searched without them)
 static __device__ __forceinline__ void res_block_sums(const float2* st, int j0, int len, double* blocks, int w, int step) {
     for (int k = w; k < len / 256 - 1; k += step) {
-        const double t = svs::block_sum([&](int j) {
+        float4 v[4];
+        svs::block_load(v, [&](int j) {
             const float2 x = st[swz(j0 + 256 * k + j)], y = st[swz(j0 + 256 * k + j + 1)];
             return make_float4(x.x, x.y, y.x, y.y);
         });
+        const double t = svs::block_sum(v);
         if ((threadIdx.x & 31) == 0) blocks[k] = t;
     }
 }

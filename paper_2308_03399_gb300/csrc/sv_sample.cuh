@@ -124,12 +124,13 @@ template <> struct Sum<float> {
     }
     __device__ __forceinline__ Sum3 wide() const { return {hi, lo, 0.f}; }
 };
-// the sum of |psi_j|^2 over 256 amplitudes, one warp, every lane; pair(j)
-// gives amplitudes j and j + 1 (j even)
-template <class Pair> __device__ __forceinline__ double block_sum(Pair pair) {
-    float4 v[4];
+// the sum of |psi_j|^2 over a block of 256 amplitudes, one warp, every lane:
+// first the lane's amplitudes, pair(j) giving j and j + 1 (j even)
+template <class Pair> __device__ __forceinline__ void block_load(float4 (&v)[4], Pair pair) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[k] = pair(2 * ((threadIdx.x & 31) + 32 * k));
+}
+__device__ __forceinline__ double block_sum(const float4 (&v)[4]) {
     Sum3 t;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -280,22 +281,36 @@ __device__ __forceinline__ int64_t sample_warp(const typename Cx<R>::T* g, int64
     if (c < chunks) {
         double acc = c ? cum[(int64_t)(c - 1) * stride] : 0.0;
         const int64_t j0 = (int64_t)c * L;
+        // (complex64) a block's amplitudes are on their way while the one
+        // before it is summed
+        float4 v[4];
+        auto load = [&](float4 (&w)[4], int64_t blk) {
+            if constexpr (sizeof(R) == 4 && !BLOCKS) {
+                const typename Cx<R>::T* gb = g + j0 + blk;
+                const bool aligned = (reinterpret_cast<uintptr_t>(gb) & 15) == 0;
+                block_load(w, [&](int j) { return load_pair(gb + j, aligned); });
+            }
+        };
+        if (L > 256) load(v, 0);
         for (int64_t blk = 0; blk < L && key < 0; blk += 256) {
             if constexpr (sizeof(R) == 4) {
                 // the block's total (some 500 float32 instructions, where
                 // float64 takes 45 of 16 clocks); the running sums below
                 // only for the block that holds the draw
-                if (L > 256) {
+                if (blk + 256 < L) {
                     double tot;
+                    float4 next[4];
                     if constexpr (BLOCKS) {
-                        tot = blk + 256 < L ? blocks[blk / 256] : 0.0;
+                        tot = blocks[blk / 256];
                     } else {
-                        const typename Cx<R>::T* gb = g + j0 + blk;
-                        const bool aligned = (reinterpret_cast<uintptr_t>(gb) & 15) == 0;
-                        tot = block_sum([&](int j) { return load_pair(gb + j, aligned); });
+                        load(next, blk + 256);
+                        tot = block_sum(v);
                     }
-                    if (!(u < acc + tot) && blk + 256 < L) {
+                    if (!(u < acc + tot)) {
                         acc += tot;
+                        if constexpr (!BLOCKS)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) v[k] = next[k];
                         continue;
                     }
                 }
