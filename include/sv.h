@@ -336,7 +336,8 @@ sv_status sv_profile(sv_batch b, double *ms, int64_t *launches);
  * plug-ins to allocate, or a latency-critical loop where cudaMalloc's
  * implicit synchronisation would stall the device.  It draws one key per
  * state exactly as sv_counts / sv_run_circuit do (same Philox draw, same
- * chunked float64 prefix), from states and into keys the caller provides:
+ * chunked prefix to float64 precision), from states and into keys the caller
+ * provides:
  *   states   device, n_states consecutive states of 2^n_qubits amplitudes
  *            (float2 for SV_C64, double2 for SV_C128), read only
  *   shots    device, n_states 64-bit global shot ids: state i draws with

@@ -15,8 +15,8 @@
 // (stage by stage, or the folded matrix where the pass was folded), so
 // without Kraus ops and measurements complex64 states are the same to the
 // last bit.  The probabilities of those are sums over the whole state, here
-// over other lanes than in a pass (float-float per lane, float64 across
-// lanes and warps in both): they agree to about 1e-14, and the factor
+// over other lanes than in a pass (float-float per lane, to float64 precision
+// across lanes and warps in both): they agree to about 1e-14, and the factor
 // 1 / sqrt(p) of a choice, rounded to float32, can come out one float32
 // rounding apart (some 1e-7 of the choices).
 //
@@ -36,12 +36,12 @@
 // meanwhile.
 //
 // Measured on GB300, us a run, passes -> resident: 6-qubit brickwork x 100
-// shots 169 -> 74, 10-qubit x 1000 829 -> 292, 13-qubit QFT x 4000 6550 ->
+// shots 169 -> 73, 10-qubit x 1000 829 -> 298, 13-qubit QFT x 4000 6550 ->
 // 2500, 12-qubit QFT with Kraus noise x 4000 (shot-branching passes) 30700 ->
-// 16700, 11-qubit complex128 sweep x 1000 2680 -> 2250.  What bounds it: issue
-// slots (42% used at 12 qubits, some 7000 warp instructions a Kraus pass) and
-// barriers in complex64, the float64 pipe (two lanes per clock per SM) in
-// complex128.
+// 17000, 11-qubit complex128 sweep x 1000 2690 -> 2260.  What bounds it:
+// barriers and latency in complex64 (47% of issue slots used at 12 qubits,
+// 6500 warp instructions a Kraus pass and state), the float64 pipe (two lanes
+// per clock per SM) in complex128.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -59,8 +59,9 @@ namespace {
 // CTA shapes: CTAs of 128 threads per SM (registers), by precision and
 // whether the circuit has folded blocks.  A spilled word costs more than the
 // warps it buys: the state takes most of the SM's memory and leaves little
-// L1 behind it (a Kraus circuit of 12 qubits ran 18.6 ms at 12 warps a SM and
-// 22 ms at 20 with 300 bytes of spills).
+// L1 behind it (a Kraus circuit of 12 qubits ran 22 ms at 20 warps a SM with
+// 300 bytes of spills and 18.6 ms at 12 with none; at 16, this, with 12 bytes,
+// 16.7 ms, each with float-float sums across lanes).
 template <class R, int NT, bool FOLDS> struct ResCta { static constexpr int min_blocks = 1; };
 template <> struct ResCta<float, 128, true> { static constexpr int min_blocks = 4; };
 template <> struct ResCta<float, 128, false> { static constexpr int min_blocks = 4; };
@@ -159,7 +160,8 @@ template <class R> __device__ __forceinline__ double res_scale(double p) {
 }
 
 // history of a shot: a sum of one mixed word per (op, outcome), so that two
-// shots with equal words took the same outcomes
+// shots with equal words took the same outcomes (the mixer and increment of
+// splitmix64: Steele, Lea, Flood, OOPSLA'14)
 __device__ __forceinline__ unsigned long long hist_word(uint32_t op, int sel) {
     unsigned long long x = ((unsigned long long)op << 32 | (uint32_t)sel) + 0x9E3779B97F4A7C15ull;
     x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;

@@ -1504,10 +1504,12 @@ sv_status circuit_op(sv_batch b, const sv_circuit* c, int i) {
     return fail(SV_EINVAL, "unknown op kind");
 }
 
-// four independent lanes of 8 bytes: a byte-wise hash's multiply chain took
-// longer than a small circuit's kernels (70 us for the 54 KB of tables of a
-// 10-qubit, depth-20 brickwork)
-uint64_t fnv(uint64_t h, const void* p, size_t n) {
+// FNV-1a (Fowler, Noll, Vo; offset basis and 64-bit prime) over the last bytes,
+// and before them four independent lanes of 8 bytes with primes of xxHash
+// (Collet) and the golden ratio as multipliers and offsets: a byte-wise hash's
+// multiply chain took longer than a small circuit's kernels (70 us for the
+// 54 KB of tables of a 10-qubit, depth-20 brickwork)
+uint64_t hash_bytes(uint64_t h, const void* p, size_t n) {
     const unsigned char* c = (const unsigned char*)p;
     uint64_t a[4] = {h, h + 0x9E3779B97F4A7C15ull, h + 0xC2B2AE3D27D4EB4Full, h + 0x165667B19E3779F9ull};
     for (; n >= 32; n -= 32, c += 32)
@@ -1525,25 +1527,25 @@ uint64_t fnv(uint64_t h, const void* p, size_t n) {
 
 uint64_t circuit_hash(sv_batch b, const sv_circuit* c) {
     uint64_t h = 1469598103934665603ull;
-    h = fnv(h, &c->n_qubits, 12);
+    h = hash_bytes(h, &c->n_qubits, 12);
     const size_t n = c->n_ops;
-    h = fnv(h, c->kind, 4 * n);
-    h = fnv(h, c->nq, 4 * n);
-    h = fnv(h, c->q_off, 4 * n);
-    h = fnv(h, c->n_terms, 4 * n);
-    h = fnv(h, c->d_off, 8 * n);
-    h = fnv(h, c->cond_clbit, 4 * n);
-    h = fnv(h, c->cond_val, 4 * n);
+    h = hash_bytes(h, c->kind, 4 * n);
+    h = hash_bytes(h, c->nq, 4 * n);
+    h = hash_bytes(h, c->q_off, 4 * n);
+    h = hash_bytes(h, c->n_terms, 4 * n);
+    h = hash_bytes(h, c->d_off, 8 * n);
+    h = hash_bytes(h, c->cond_clbit, 4 * n);
+    h = hash_bytes(h, c->cond_val, 4 * n);
     // (arrays that only measurements have may be NULL without one; what
     // op_measure refuses is not read)
     for (size_t i = 0; i < n; ++i)
         if (c->kind[i] == SV_OP_MEASURE && c->nq[i] >= 1 && c->nq[i] <= 4 && c->clbits) {
-            h = fnv(h, c->clbits + c->cl_off[i], 4 * (size_t)c->nq[i]);
-            h = fnv(h, c->reset + i, 4);
+            h = hash_bytes(h, c->clbits + c->cl_off[i], 4 * (size_t)c->nq[i]);
+            h = hash_bytes(h, c->reset + i, 4);
         }
     int64_t dmax = 0, qmax = 0;
     for (size_t i = 0; i < n; ++i) qmax = std::max<int64_t>(qmax, c->q_off[i] + c->nq[i]);
-    h = fnv(h, c->qubits, 4 * qmax);
+    h = hash_bytes(h, c->qubits, 4 * qmax);
     for (size_t i = 0; i < n; ++i) {
         const int k = c->nq[i];
         int64_t len = 0;
@@ -1552,10 +1554,10 @@ uint64_t circuit_hash(sv_batch b, const sv_circuit* c) {
         else if (c->kind[i] == SV_OP_KRAUS || c->kind[i] == SV_OP_PGATE) len = (int64_t)c->n_terms[i] * (2ll << (2 * k));
         dmax = std::max<int64_t>(dmax, c->d_off[i] + len);
     }
-    h = fnv(h, c->data, 8 * dmax);
+    h = hash_bytes(h, c->data, 8 * dmax);
     for (size_t i = 0; i < n; ++i)
-        if (c->kind[i] == SV_OP_PAULI) h = fnv(h, c->paulis + c->s_off[i], (size_t)c->n_terms[i] * c->nq[i]);
-    h = fnv(h, &b->mode, sizeof(b->mode));
+        if (c->kind[i] == SV_OP_PAULI) h = hash_bytes(h, c->paulis + c->s_off[i], (size_t)c->n_terms[i] * c->nq[i]);
+    h = hash_bytes(h, &b->mode, sizeof(b->mode));
     return h;
 }
 
@@ -2182,10 +2184,15 @@ bool build_resident(sv_batch b, std::vector<Launch>& launches) {
     memset(&r, 0, sizeof(r));
     r.np = std::max(4, b->n);
     // states that leave room for one CTA per SM: its latency is hidden by
-    // nothing else, so over many waves passes with a reduction come out even
-    // and complex128 ones behind (14-qubit SU(4), 100 shots 4.06 ms on passes
-    // and 0.70 resident, 2000 shots 9.5 and 8.9; 13-qubit complex128
-    // mid-circuit measurements, 100 shots 7.4 and 1.9 ms, 2000 21.4 and 25.5)
+    // nothing else, so over many waves passes with a reduction come out ahead
+    // or behind by the circuit (14 qubits x 4000, passes and resident: SU(4)
+    // 7.2 and 8.4 ms, mid-circuit measurements 5.8 and 5.1, QFT with Kraus
+    // noise 117 and 98; x 700 2.1 and 1.6, 1.36 and 0.96, 39 and 18) and
+    // complex128 ones behind (13 qubits x 2000: brickwork 24.9 and 27.1 ms,
+    // mid-circuit measurements 12.4 and 13.1).  Two CTAs per SM stay ahead or
+    // even (12 qubits, complex128, x 4000: brickwork 22.7 and 23.0, SU(4) 25.9
+    // and 24.9, mid-circuit measurements 11.2 and 10.3; x 700 4.5 and 4.3, 5.8
+    // and 4.7, 2.4 and 2.0).
     if (resident_one_cta(b->prec == SV_C128, r.np) && b->n_shots > (uint64_t)4 * b->n_sm) {
         bool red = b->prec == SV_C128;
         for (const Launch& L : launches) red = red || (L.type == L_PASS && L.pass.red_kind != RED_NONE);
@@ -2289,7 +2296,7 @@ sv_status fold_histories(sv_batch b) {
 sv_status note_run(sv_batch b, uint64_t hash, bool resident) {
     b->res_branch_last = b->branch && resident;
     if (!b->res_branch_last) return SV_OK;
-    const uint64_t key = fnv(hash, &b->pool_gen, 8);
+    const uint64_t key = hash_bytes(hash, &b->pool_gen, 8);
     if (key != b->res_key)
         if (sv_status st = fold_histories(b)) return st;
     b->res_key = key;
@@ -2956,8 +2963,8 @@ sv_status sv_run_circuits(sv_batch* bs, const sv_circuit* const* cs, int n, int 
     uint64_t h = 1469598103934665603ull;
     for (int i = 0; i < n; ++i) {
         const uint64_t hi = circuit_hash(bs[i], cs[i]);
-        h = fnv(h, &hi, 8);
-        h = fnv(h, &bs[i], sizeof(void*));
+        h = hash_bytes(h, &hi, 8);
+        h = hash_bytes(h, &bs[i], sizeof(void*));
     }
     bool cached = use_graph && b0->multi_exec && b0->multi_hash == h && (int)b0->multi_gens.size() == n;
     for (int i = 0; cached && i < n; ++i) cached = b0->multi_gens[i] == bs[i]->pool_gen;

@@ -30,7 +30,8 @@ DEFAULT = dict(mode="branch", max_active=0, path=0, joint=1, tile=0)  # the libr
 # A pick leaves the defaults only for a predicted time below this share of
 # theirs: they are the only configuration that runs small registers as one
 # resident launch (a step in time that a smooth model rounds off), and over
-# the 36 circuits of the timing log they take 1.15x the per-circuit best
+# the 36 circuits of the timing log, on which this share was chosen, they take
+# 1.15x the per-circuit best
 LEAVE_DEFAULT = 0.7
 
 
